@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kTailThreads) k_tail(TailArgs<T> a, const int*
         cNW[q] = G.cNW[k];
         dg[q] = G.diag[k];
         di[q] = G.dinv[k];
-        xs[q] = (l == 0) ? a.lv[0].x[k] : T(0);
+        xs[q] = (l == 0 && !a.zero) ? a.lv[0].x[k] : T(0);
         bsm[q] = (l == 0) ? a.lv[0].b[k] : T(0);
       }
     }

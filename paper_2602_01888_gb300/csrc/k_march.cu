@@ -36,6 +36,7 @@
 #include "mg_common.cuh"
 #include "mg_launch.h"
 #include "mg_march.h"
+#include "mg_block.h"
 #include "mg_tile.h"
 
 namespace mg {
@@ -560,10 +561,26 @@ __global__ void __launch_bounds__(MarchGeom<T, CFG>::THREADS, MarchGeom<T, CFG>:
   }
 }
 
-// Variants: the configurations of MarchGeom; variant 0 is each precision's default.
+// Variants: kMarchCfg gives the configuration of MarchGeom, or -ns for a register-block pass of ns
+// sweeps (k_block.cu).  Variant 0 is each precision's default: FP32 the register blocks, FP64
+// configuration 3.
+constexpr int kMarchCfgF32[] = {-2, 0, 1, 2, 3, 4};
+constexpr int kMarchCfgF64[] = {3, 1, 2, 0, -1};
+
 template <typename T>
 int march_variants() {
-  return sizeof(T) == 8 ? 4 : 5;
+  return sizeof(T) == 8 ? (int)(sizeof(kMarchCfgF64) / sizeof(int)) : (int)(sizeof(kMarchCfgF32) / sizeof(int));
+}
+
+template <typename T>
+static int march_cfg_of(int v) {
+  if (v < 0 || v >= march_variants<T>()) v = 0;
+  return sizeof(T) == 8 ? kMarchCfgF64[v] : kMarchCfgF32[v];
+}
+
+template <typename T>
+bool march_in_blocks(int v) {
+  return march_cfg_of<T>(v) < 0;
 }
 
 template <typename T, int CFG>
@@ -571,27 +588,19 @@ static SmoothVariant march_cfg() {
   return {MarchGeom<T, CFG>::W, 0, MarchGeom<T, CFG>::NS};
 }
 
-// FP64 variant -> configuration: variant 0 (the default) is configuration 3, measured the
-// fastest at 2049^2-8193^2 (1.46 ms a sweep at 8193^2 against 1.69 for configuration 2 and
-// 2.26 for configuration 0, whose four compute warps leave the FP64 pipe waiting on their
-// dependent FMA chains).
-static int f64_cfg(int v) {
-  constexpr int cfg[4] = {3, 1, 2, 0};
-  return cfg[(v < 0 || v >= 4) ? 0 : v];
-}
-
 template <typename T>
 SmoothVariant march_variant(int v) {
-  if (v < 0 || v >= march_variants<T>()) v = 0;
+  const int cfg = march_cfg_of<T>(v);
+  if (cfg < 0) return {block_tile_width<T>(-cfg), 0, -cfg};
   if constexpr (sizeof(T) == 8) {
-    switch (f64_cfg(v)) {
+    switch (cfg) {
       case 1: return march_cfg<double, 1>();
       case 2: return march_cfg<double, 2>();
       case 3: return march_cfg<double, 3>();
       default: return march_cfg<double, 0>();
     }
   } else {
-    switch (v) {
+    switch (cfg) {
       case 1: return march_cfg<float, 1>();
       case 2: return march_cfg<float, 2>();
       case 3: return march_cfg<float, 3>();
@@ -671,16 +680,24 @@ static cudaError_t march_impl(const Op<T>& A, const T* xin, T* xout, const T* b,
 template <typename T>
 cudaError_t launch_smooth_march(const Op<T>& A, const T* xin, T* xout, const T* b, int rev,
                                 const T* eH, int pitch_c, const int* skip, cudaStream_t s, int v) {
-  if (v < 0 || v >= march_variants<T>()) v = 0;
+  const int cfg = march_cfg_of<T>(v);
+  if (cfg < 0) {  // the family's requirements on pitch and alignment hold for every variant
+    constexpr int VEC = 16 / (int)sizeof(T);
+    if (A.pitch % VEC != 0 || (eH && pitch_c % VEC != 0)) return cudaErrorInvalidValue;
+    if (((uintptr_t)xin | (uintptr_t)xout | (uintptr_t)b | (uintptr_t)A.cE | (uintptr_t)A.cN |
+         (uintptr_t)A.cNE | (uintptr_t)A.cNW | (uintptr_t)A.dinv | (uintptr_t)eH) % 16 != 0)
+      return cudaErrorInvalidValue;
+    return launch_smooth_block<T>(A, xin, xout, b, -cfg, rev, eH, nullptr, pitch_c, skip, s);
+  }
   if constexpr (sizeof(T) == 8) {
-    switch (f64_cfg(v)) {
+    switch (cfg) {
       case 1: return march_impl<double, 1>(A, xin, xout, b, rev, eH, pitch_c, skip, s);
       case 2: return march_impl<double, 2>(A, xin, xout, b, rev, eH, pitch_c, skip, s);
       case 3: return march_impl<double, 3>(A, xin, xout, b, rev, eH, pitch_c, skip, s);
       default: return march_impl<double, 0>(A, xin, xout, b, rev, eH, pitch_c, skip, s);
     }
   } else {
-    switch (v) {
+    switch (cfg) {
       case 1: return march_impl<float, 1>(A, xin, xout, b, rev, eH, pitch_c, skip, s);
       case 2: return march_impl<float, 2>(A, xin, xout, b, rev, eH, pitch_c, skip, s);
       case 3: return march_impl<float, 3>(A, xin, xout, b, rev, eH, pitch_c, skip, s);
@@ -690,6 +707,8 @@ cudaError_t launch_smooth_march(const Op<T>& A, const T* xin, T* xout, const T* 
   }
 }
 
+template bool march_in_blocks<float>(int);
+template bool march_in_blocks<double>(int);
 template int march_sweeps<float>(int);
 template int march_sweeps<double>(int);
 template int march_strip_width<float>(int);

@@ -26,6 +26,7 @@ struct TailLevel {
 template <typename T>
 struct TailArgs {
   int nlev, nu1, nu2;
+  int zero;  // 1: the finest level's iterate starts from zero (x is not read)
   int line;  // 1: zebra x-line Gauss-Seidel on the tail levels, 0: four-colour Gauss-Seidel
   const double* inv;
   TailLevel<T> lv[kMaxTail];

@@ -12,6 +12,9 @@ template <typename T>
 int march_sweeps(int v = -1);
 template <typename T>
 int march_strip_width(int v = -1);
+// Whether variant v is the register-block kernel (k_block.cu), which takes levels of any height.
+template <typename T>
+bool march_in_blocks(int v = -1);
 
 // xout = march_sweeps<T>(v) Gauss-Seidel sweeps of (xin [+ P eH]) in forward (rev = 0) or
 // reversed colour order; xin != xout; every array 16-byte aligned, pitch a multiple of

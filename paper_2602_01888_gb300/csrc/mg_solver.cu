@@ -787,7 +787,6 @@ static mg_status emit_body(mg_problem* P, const mg_solve_opts& o, cudaGraphCondi
     } else {
       CU(launch_resid_check(F.A, F.x, F.b, P->r, P->st, P->part, h, has_h, s));
       CU(launch_r_to_f32(F.A, P->r, F.b32, F.A32.pitch, P->st, s));
-      if (vcycle_reads_x0(o.smoother, o.nu1)) CU(cudaMemsetAsync(F.x32, 0, n0 * sizeof(float), s));
       float* res = nullptr;
       if ((st = emit_vcycle_on<float>(P, F.x32, F.b32, o, skip, s, &res, true))) return st;
       CU(launch_add_f32(F.A, F.x, res, F.A32.pitch, P->st, s));
@@ -800,13 +799,11 @@ static mg_status emit_body(mg_problem* P, const mg_solve_opts& o, cudaGraphCondi
   CU(launch_fcg_verify(F.A, F.x, F.b, P->r, mixed ? F.b32 : nullptr, F.A32.pitch, P->st, P->part, h,
                        has_h, s));
   if (!mixed) {
-    if (vcycle_reads_x0(o.smoother, o.nu1)) CU(cudaMemsetAsync(P->z, 0, n0 * sizeof(double), s));
     double* res = nullptr;
     if ((st = emit_vcycle_on<double>(P, P->z, P->r, o, skip, s, &res, true))) return st;
     CU(launch_fcg_zq<double>(F.A, res, F.A.pitch, P->q, P->st, P->part, s));
     CU(launch_fcg_pq<double>(F.A, res, F.A.pitch, P->p, P->q, P->r, P->st, P->part, s));
   } else {
-    if (vcycle_reads_x0(o.smoother, o.nu1)) CU(cudaMemsetAsync(F.x32, 0, n0 * sizeof(float), s));
     float* res = nullptr;
     if ((st = emit_vcycle_on<float>(P, F.x32, F.b32, o, skip, s, &res, true))) return st;
     CU(launch_fcg_zq<float>(F.A, res, F.A32.pitch, P->q, P->st, P->part, s));

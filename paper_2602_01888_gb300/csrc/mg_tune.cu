@@ -77,7 +77,7 @@ static float time_family(mg_ctx* ctx, int kind, int v, const Op<T>& A, T* x, T* 
   // the same applicability rules as the cycle
   if (kind != SK_COLOUR && 2 % ns) return -1.f;
   if (kind == SK_PIPE && (nyr < 64 || A.nx < 160)) return -1.f;
-  if (kind == SK_MARCH && nyr < 128) return -1.f;
+  if (kind == SK_MARCH && nyr < 128 && !march_in_blocks<T>(v)) return -1.f;
   for (int w = 0; w < 2; ++w)
     if (once() != cudaSuccess) return -1.f;
   cudaEvent_t e0, e1;

@@ -1,8 +1,9 @@
 // One multigrid V(nu1, nu2) cycle (Sec. 3, Eqs. 19-24) enqueued on a stream.  Smoothing
-// per level, by size: the largest levels use the row-marching kernel (FP32 two sweeps a
-// pass, FP64 one), other large FP32 levels the pipelined tile kernel, other large FP64
-// levels the per-colour kernels, mid-size levels the fused tile kernel (NS sweeps per launch,
-// ping-pong iterates); the residual is fused with full-weighting restriction; the levels
+// per level: FP32 levels of aligned rows use the register-block kernel (two sweeps a pass, started
+// from zero without reading the iterate, the last pre-smoothing pass fused with the residual and
+// its full weighting); FP64 levels by size the row-marching kernel, the per-colour kernels or the
+// fused tile kernel (NS sweeps per launch, ping-pong iterates), then one kernel for the residual
+// fused with full-weighting restriction; the levels
 // at and below the tail threshold run in one single-CTA tail kernel that ends with the
 // coarsest dense solve.  The weighted-Jacobi smoother uses the per-sweep kernels on every
 // level, the zebra x-line smoother its two launches a sweep on every level but the coarsest.
@@ -11,6 +12,7 @@
 #include <cstring>
 
 #include "mg.h"
+#include "mg_block.h"
 #include "mg_fused.h"
 #include "mg_internal_host.h"
 #include "mg_kernels.h"
@@ -108,7 +110,10 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
     alt[l] = V.t[l];
   }
   cudaError_t e;
+  auto level_bytes = [&](int l) { return (size_t)V.A[l].pitch * rows_stored(V.A[l].ny, V.A[l].periodic) * sizeof(T); };
+  auto clear = [&](int l) { return cudaMemsetAsync(cur[l], 0, level_bytes(l), s); };
   if (smoother == MG_SMOOTH_JACOBI) {
+    if (x0_zero && (e = clear(0))) return e;
     for (int l = 0; l < L - 1; ++l) {
       if ((e = launch_jacobi(V.A[l], cur[l], V.b[l], alt[l], nu1, omega, skip, s))) return e;
       if ((e = launch_resid_restrict(V.A[l], cur[l], V.b[l], V.b[l + 1], cur[l + 1],
@@ -133,6 +138,7 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
     // memory) run with the coarsest solve in the single-CTA tail kernel, which smooths them
     // row by row: one launch instead of about six per level, each of them latency-bound.
     const bool zs = nu1 > 0;
+    if (x0_zero && !zs && (e = clear(0))) return e;
     int t = L - 1;
     const int thr = line_tail_nodes<T>();
     for (int l = 1; l < L - 1; ++l) {
@@ -149,10 +155,10 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
       const int zero = l == 0 ? (x0_zero && zs) : zs;
       if ((e = launch_line_smooth(V.A[l], V.lf[l], cur[l], V.b[l], nu1, 0, skip, s, (const T*)nullptr, 0, zero)))
         return e;
-      // the tail kernel reads the iterate of its first level: clear it there.  After
-      // pre-smoothing, whose last half-sweep solved the odd rows, only the even rows'
-      // residual is restricted (launch_resid_restrict_even).
-      T* const xc = zs && l + 1 < t ? nullptr : cur[l + 1];
+      // without pre-smoothing a coarse level's iterate is read, so it is cleared here (the tail
+      // kernel starts from zero by itself).  After pre-smoothing, whose last half-sweep solved
+      // the odd rows, only the even rows' residual is restricted (launch_resid_restrict_even).
+      T* const xc = zs || l + 1 == t ? nullptr : cur[l + 1];
       if ((e = zs ? launch_resid_restrict_even(V.A[l], cur[l], V.b[l], V.b[l + 1], xc, V.A[l + 1].pitch, skip, s)
                   : launch_resid_restrict(V.A[l], cur[l], V.b[l], V.b[l + 1], xc, V.A[l + 1].pitch, skip, s)))
         return e;
@@ -165,6 +171,7 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
       ta.nlev = L - t;
       ta.nu1 = nu1;
       ta.nu2 = nu2;
+      ta.zero = 1;
       ta.line = 1;
       ta.inv = V.inv;
       for (int l = t; l < L; ++l) {
@@ -203,15 +210,16 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
     }
   }
   const long long cthr = colour_nodes<T>();
-  auto smooth = [&](int l, int sweeps, int rev, const T* eH) -> cudaError_t {
-    cudaError_t err;
+  // smoother family and variant of level l for this many sweeps
+  auto choose = [&](int l, int sweeps, int* var_out) -> int {
     const long long nodes = (long long)V.A[l].nx * rows_stored(V.A[l].ny, V.A[l].periodic);
     const int nyr = rows_stored(V.A[l].ny, V.A[l].periodic);
-    const int pc = eH ? V.A[l + 1].pitch : 0;
     // which families (in a given variant) can run this level with this many sweeps
     auto can = [&](int kind, int v) {
       if (sweeps <= 0) return kind == SK_COLOUR;
       switch (kind) {
+        case SK_BLOCK:
+          return block_can(V.A[l], V.x[l], V.t[l], V.b[l]);
         case SK_MARCH:
           return sweeps % march_sweeps<T>(v) == 0 && V.A[l].pitch % (16 / (int)sizeof(T)) == 0 && nyr >= 128;
         case SK_PIPE:
@@ -224,9 +232,12 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
           return kind == SK_COLOUR;
       }
     };
-    // size-threshold rule, default variants
+    // size-threshold rule, default variants.  FP32: register blocks were the fastest at every size
+    // from 65^2 to 4097^2 (figures in k_block.cu), so size does not enter
     int kind, var = -1;
-    if (nodes >= march_nodes() && can(SK_MARCH, -1))
+    if (sizeof(T) == 4 && can(SK_BLOCK, -1))
+      kind = SK_BLOCK;
+    else if (sizeof(T) == 8 && nodes >= march_nodes() && can(SK_MARCH, -1))
       kind = SK_MARCH;
     else if (sizeof(T) == 4 && nodes > cthr && can(SK_PIPE, -1))
       kind = SK_PIPE;
@@ -237,17 +248,42 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
     // measured choice, where it can run
     if (V.pol) {
       int v = -1;
-      const int k = V.pol->lookup(nodes, &v);
+      int k = V.pol->lookup(nodes, &v);
+      if (k == SK_MARCH && march_in_blocks<T>(v)) k = SK_BLOCK;
       if (k != SK_DEFAULT && can(k, v)) {
         kind = k;
         var = v;
       }
     }
+    *var_out = var;
+    return kind;
+  };
+  // `sweeps` sweeps of level l.  eH: after adding the coarse correction.  zero: from a zero
+  // iterate, which cur[l] need not hold if starts_blind(l).  bH: and the restricted residual of
+  // the result; xH (nullable): a coarse iterate to clear.
+  auto smooth = [&](int l, int sweeps, int rev, const T* eH, bool zero, T* bH, T* xH) -> cudaError_t {
+    cudaError_t err;
+    const int pc = l + 1 < L ? V.A[l + 1].pitch : 0;
+    int var = -1;
+    const int kind = choose(l, sweeps, &var);
     auto swap_cur = [&]() {
       T* tmp = cur[l];
       cur[l] = alt[l];
       alt[l] = tmp;
     };
+    if (kind == SK_BLOCK) {  // passes of block_sweeps<T>() sweeps, an odd one first
+      constexpr int NB = block_sweeps<T>();
+      for (int left = sweeps; left > 0;) {
+        const int ns = left % NB ? 1 : NB;
+        const bool first = left == sweeps, last = left == ns;
+        err = launch_smooth_block<T>(V.A[l], first && zero ? nullptr : cur[l], alt[l], V.b[l], ns, rev,
+                                     first ? eH : nullptr, last ? bH : nullptr, pc, skip, s);
+        if (err) return err;
+        swap_cur();
+        left -= ns;
+      }
+      return xH ? clear(l + 1) : cudaSuccess;
+    }
     if (kind == SK_MARCH) {
       for (int k = 0; k < sweeps / march_sweeps<T>(var); ++k) {
         err = launch_smooth_march<T>(V.A[l], cur[l], alt[l], V.b[l], rev, k == 0 ? eH : nullptr, pc, skip, s,
@@ -255,41 +291,42 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
         if (err) return err;
         swap_cur();
       }
-      return cudaSuccess;
-    }
-    if (kind == SK_PIPE) {
+    } else if (kind == SK_PIPE) {
       for (int k = 0; k < sweeps / pipe_sweeps<T>(var); ++k) {
         err = launch_smooth_pipe<T>(V.A[l], cur[l], alt[l], V.b[l], rev, k == 0 ? eH : nullptr, pc, skip,
                                     V.err, s, var);
         if (err) return err;
         swap_cur();
       }
-      return cudaSuccess;
-    }
-    if (kind == SK_COLOUR) {  // per-colour kernels, in place
+    } else if (kind == SK_COLOUR) {  // per-colour kernels, in place
       if (eH && (err = launch_prolong_add(V.A[l], cur[l], eH, pc, skip, s))) return err;
-      return launch_smooth(V.A[l], cur[l], V.b[l], sweeps, rev, skip, s);
+      if ((err = launch_smooth(V.A[l], cur[l], V.b[l], sweeps, rev, skip, s))) return err;
+    } else {
+      for (int k = 0; k < sweeps / fused_sweeps<T>(var); ++k) {
+        err = launch_smooth_fused(V.A[l], cur[l], alt[l], V.b[l], rev, k == 0 ? eH : nullptr, pc, skip, s, var);
+        if (err) return err;
+        swap_cur();
+      }
     }
-    for (int k = 0; k < sweeps / fused_sweeps<T>(var); ++k) {
-      err = launch_smooth_fused(V.A[l], cur[l], alt[l], V.b[l], rev, k == 0 ? eH : nullptr, pc, skip, s, var);
-      if (err) return err;
-      swap_cur();
-    }
-    if (sweeps == 0 && eH) return launch_prolong_add(V.A[l], cur[l], eH, pc, skip, s);
-    return cudaSuccess;
+    return bH ? launch_resid_restrict(V.A[l], cur[l], V.b[l], bH, xH, pc, skip, s) : cudaSuccess;
   };
-  for (int l = 0; l < t; ++l) {
-    if ((e = smooth(l, nu1, 0, nullptr))) return e;
-    if ((e = launch_resid_restrict(V.A[l], cur[l], V.b[l], V.b[l + 1], cur[l + 1], V.A[l + 1].pitch,
-                                   skip, s)))
+  // whether level l's pre-smoothing from a zero iterate leaves the stored one unread
+  auto starts_blind = [&](int l) {
+    int v;
+    return nu1 > 0 && choose(l, nu1, &v) == SK_BLOCK;
+  };
+  if (t > 0 && x0_zero && !starts_blind(0) && (e = clear(0))) return e;
+  for (int l = 0; l < t; ++l)  // the tail kernel starts from zero by itself
+    if ((e = smooth(l, nu1, 0, nullptr, l > 0 || x0_zero, V.b[l + 1],
+                    l + 1 < t && !starts_blind(l + 1) ? cur[l + 1] : nullptr)))
       return e;
-  }
   {
     TailArgs<T> ta;
     memset(&ta, 0, sizeof ta);
     ta.nlev = L - t;
     ta.nu1 = nu1;
     ta.nu2 = nu2;
+    ta.zero = t > 0 || x0_zero;
     ta.inv = V.inv;
     for (int l = t; l < L; ++l) {
       ta.lv[l - t].L = lvl_of(V.A[l]);
@@ -300,7 +337,7 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
     if ((e = launch_tail(ta, skip, s))) return e;
   }
   for (int l = t - 1; l >= 0; --l)
-    if ((e = smooth(l, nu2, 1, cur[l + 1]))) return e;
+    if ((e = smooth(l, nu2, 1, cur[l + 1], false, nullptr, nullptr))) return e;
   *result = cur[0];
   return cudaSuccess;
 }

@@ -10,8 +10,9 @@ namespace mg {
 constexpr int kMaxVLevels = 24;
 
 // Smoother family for a level: the per-colour kernels (four launches a sweep), the fused
-// tile kernel, the pipelined tile kernel, the row-marching kernel.
-enum SmoothKind : int { SK_DEFAULT = 0, SK_COLOUR = 1, SK_FUSED = 2, SK_PIPE = 3, SK_MARCH = 4 };
+// tile kernel, the pipelined tile kernel, the row-marching kernel, the register-block kernel (to
+// the autotuner a variant of the marching family).
+enum SmoothKind : int { SK_DEFAULT = 0, SK_COLOUR = 1, SK_FUSED = 2, SK_PIPE = 3, SK_MARCH = 4, SK_BLOCK = 5 };
 
 // Measured choice of smoother family and variant by level size (filled by mg_autotune):
 // entry k says that square levels of side[k] smooth fastest with kind[k], variant var[k] (tile
@@ -42,17 +43,12 @@ struct VLevels {
 };
 
 // Enqueue one V(nu1, nu2) cycle starting from the iterate in V.x[0]; *result receives the
-// array (V.x[0] or V.t[0]) that holds the level-0 result.  x0_zero: the caller's iterate is
-// zero at every unknown (the preconditioner's start) and its Dirichlet nodes are zero, so a
-// smoother that can use it need not read it (the caller may skip clearing it when
-// vcycle_reads_x0() says so).
+// array (V.x[0] or V.t[0]) that holds the level-0 result.  x0_zero: the cycle starts from zero
+// (unknowns and Dirichlet nodes; the preconditioner's start) whatever V.x[0] holds: the first
+// smoothing pass does not read it where its kernel can do without, else it is cleared first.
 template <typename T>
 cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, double omega,
                         const int* skip, cudaStream_t s, T** result, bool x0_zero = false);
-
-// Whether emit_vcycle with x0_zero reads the unknowns of V.x[0]: false for the line
-// smoother with pre-smoothing, whose first half-sweep starts from zero without reading.
-inline bool vcycle_reads_x0(int smoother, int nu1) { return !(smoother == 2 && nu1 > 0); }
 
 template <typename T>
 int tail_nodes();
