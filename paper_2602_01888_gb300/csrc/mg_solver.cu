@@ -624,9 +624,7 @@ extern "C" mg_status mg_setup_transform(mg_ctx* ctx, const mg_grid_desc* grid,
   if (st) {
     char keep[512];
     snprintf(keep, sizeof keep, "%s", g_err);
-    cudaStreamSynchronize(ctx->stream);
-    problem_release(P);
-    delete P;
+    mg_problem_free(P);  // and out of the context's list, which mg_destroy walks
     return set_error(st, "%s", keep);
   }
   *out = P;
