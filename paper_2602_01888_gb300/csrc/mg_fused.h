@@ -46,6 +46,12 @@ cudaError_t launch_smooth_fused(const Op<T>& A, const T* xin, T* xout, const T* 
 template <typename T>
 cudaError_t launch_tail(const TailArgs<T>& a, const int* skip, cudaStream_t s);
 
+// The same in registers (k_tail.cu) for point-smoothed levels that fit it.
+template <typename T>
+bool tail_block_can(const TailArgs<T>& a);
+template <typename T>
+cudaError_t launch_tail_block(const TailArgs<T>& a, const int* skip, cudaStream_t s);
+
 // Shared-memory bytes the tail kernel needs for these levels.
 template <typename T>
 size_t tail_bytes(const TailArgs<T>& a);

@@ -334,7 +334,7 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
       ta.lv[l - t].b = V.b[l];
       ta.lv[l - t].t = alt[l];
     }
-    if ((e = launch_tail(ta, skip, s))) return e;
+    if ((e = tail_block_can(ta) ? launch_tail_block(ta, skip, s) : launch_tail(ta, skip, s))) return e;
   }
   for (int l = t - 1; l >= 0; --l)
     if ((e = smooth(l, nu2, 1, cur[l + 1], false, nullptr, nullptr))) return e;
