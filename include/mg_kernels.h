@@ -239,7 +239,8 @@ int mgk_smooth_variant_f32(const mgk_op_f32 *A, int family, int variant, const f
  * on A only:
  *   mgk_line_factor_elems(nx, ny, periodic): elements (of the operator's precision) that
  *     the factors of an nx x ny level take; 0 for sizes below 3;
- *   mgk_line_factor_*: fills `factors` for every row of A; call it again when A changes;
+ *   mgk_line_factor_*: fills `factors` for every row of A; call it again when A changes
+ *     (FP32 rows of up to 4096 unknowns are factored as they are solved: nothing is written);
  *   mgk_line_rows_*: one half-sweep of parity 0 or 1, phi updated in place;
  *   mgk_line_smooth_*: `sweeps` sweeps, each parity 0 then 1 (reverse != 0: 1 then 0).
  * Rows of up to 8192 unknowns in FP64 and 16384 in FP32 (shared-memory bound); longer

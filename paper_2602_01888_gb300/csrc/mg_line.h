@@ -27,6 +27,11 @@ size_t line_factor_elems(int nx, int ny, int periodic);
 template <typename T>
 bool line_supported(int nx);
 
+// Whether half-sweeps of a level of width nx read stored factors (FP64 always; FP32 only long rows:
+// shorter ones are factored as they are solved, and launch_line_factor writes nothing).
+template <typename T>
+bool line_stores_factors(int nx);
+
 // View of the factors of an nx x ny level stored from `base`.
 template <typename T>
 LineFactors<T> line_factors_at(T* base, int nx, int ny, int periodic);

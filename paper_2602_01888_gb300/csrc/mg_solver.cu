@@ -302,38 +302,52 @@ static mg_status problem_alloc(mg_problem* P, bool mixed) {
   return MG_OK;
 }
 
-// Line-smoother factors: levels 0 .. nlev-2 back to back, in the precision of the cycle
-// (FP32 for the mixed path).
+// Line-smoother factors of the levels above the coarsest that store them (line_stores_factors),
+// back to back, in the precision of the cycle (FP32 for the mixed path).
 template <typename T>
-static T* line_base(const mg_problem* P, int l) {
-  T* p = (T*)P->line;
-  for (int q = 0; q < l; ++q) p += line_factor_elems<T>(P->nxs[q], P->nys[q], P->grid.periodic_y);
-  return p;
+static size_t line_elems(const mg_problem* P, int l) {
+  return line_stores_factors<T>(P->nxs[l]) ? line_factor_elems<T>(P->nxs[l], P->nys[l], P->grid.periodic_y) : 0;
+}
+
+template <typename T>
+static size_t line_offset(const mg_problem* P, int l) {
+  size_t n = 0;
+  for (int q = 0; q < l; ++q) n += line_elems<T>(P, q);
+  return n;
 }
 
 template <typename T>
 static LineFactors<T> line_level(const mg_problem* P, int l) {
-  return line_factors_at<T>(line_base<T>(P, l), P->nxs[l], P->nys[l], P->grid.periodic_y);
+  if (!line_elems<T>(P, l)) return LineFactors<T>();
+  return line_factors_at<T>((T*)P->line + line_offset<T>(P, l), P->nxs[l], P->nys[l], P->grid.periodic_y);
 }
 
-static mg_status line_enqueue_factor(mg_problem* P, cudaStream_t s) {
+template <typename T>
+static mg_status line_enqueue_factor(mg_problem* P, cudaStream_t s, int* kernels) {
   for (int l = 0; l < P->nlev - 1; ++l) {
-    if (P->mixed) CU(launch_line_factor<float>(P->lev[l].A32, line_level<float>(P, l), s));
+    if (!line_elems<T>(P, l)) continue;
+    if constexpr (sizeof(T) == 4) CU(launch_line_factor<float>(P->lev[l].A32, line_level<float>(P, l), s));
     else CU(launch_line_factor<double>(P->lev[l].A, line_level<double>(P, l), s));
+    ++*kernels;
   }
   return MG_OK;
 }
 
+static mg_status line_enqueue_factor(mg_problem* P, cudaStream_t s, int* kernels) {
+  return P->mixed ? line_enqueue_factor<float>(P, s, kernels) : line_enqueue_factor<double>(P, s, kernels);
+}
+
 mg_status line_prepare(mg_problem* P, cudaStream_t s) {
   if (P->line || P->nlev < 2) return MG_OK;
-  const size_t esz = P->mixed ? sizeof(float) : sizeof(double);
-  size_t elems = 0;
-  for (int l = 0; l < P->nlev - 1; ++l) elems += line_factor_elems<double>(P->nxs[l], P->nys[l], P->grid.periodic_y);
-  void* p = P->ctx->pool.alloc(elems * esz);
+  const size_t bytes = P->mixed ? line_offset<float>(P, P->nlev - 1) * sizeof(float)
+                                : line_offset<double>(P, P->nlev - 1) * sizeof(double);
+  if (!bytes) return MG_OK;
+  void* p = P->ctx->pool.alloc(bytes);
   if (!p) return set_error(MG_ERR_OOM, "device memory budget exhausted (line-smoother factors)");
   P->allocs.push_back(p);
   P->line = p;
-  return line_enqueue_factor(P, s);
+  int kernels = 0;
+  return line_enqueue_factor(P, s, &kernels);
 }
 
 // Whether a map's transformed tensor has no cross term (Eq. 13 vanishes identically; the
@@ -494,9 +508,8 @@ mg_status problem_enqueue_build(mg_problem* P, const mg_map_desc* map, const dou
                 (P->mirror ? 1 : 0);
   if (five_pass) P->setup_kernels -= f32_done ? 2 : 1;  // one kernel for two (three with the FP32 copy)
   if (P->line) {  // the line smoother's row factors follow the new operators
-    mg_status ls = line_enqueue_factor(P, s);
+    mg_status ls = line_enqueue_factor(P, s, &P->setup_kernels);
     if (ls) return ls;
-    P->setup_kernels += P->nlev - 1;
   }
   // restore the scratch vectors used as staging (solves rely on their zero Dirichlet entries)
   if (eps_phys || map->kind == MG_MAP_GRID || P->mirror)
