@@ -99,6 +99,18 @@ __device__ void decide(SolveState* st, double rr, cudaGraphConditionalHandle h, 
   if (has_h) cudaGraphSetConditional(h, done ? 0u : 1u);
 }
 
+// Close a pass of the solve loop, by one thread of its last kernel: counts it, ends the loop after
+// 2 max_iters + 8 passes even if no decision was reached (status: not converged), and sets the
+// graph's loop condition.
+__device__ void end_of_pass(SolveState* st, cudaGraphConditionalHandle h, int has_h) {
+  st->guard += 1;
+  if (!st->done && st->guard > 2 * st->max_iters + 8) {
+    st->done = 1;
+    st->status = 6;
+  }
+  if (has_h) cudaGraphSetConditional(h, st->done ? 0u : 1u);
+}
+
 // x: Dirichlet ring from bc (or 0), unknowns from the warm start (or 0); b = rho' D (Eq. 11).
 __global__ void __launch_bounds__(kNT) k_solve_init(Lvl<double> L, const SolveArgs* __restrict__ a,
                                                     const double* __restrict__ D,
@@ -140,9 +152,9 @@ __global__ void __launch_bounds__(kNT) k_solve_init(Lvl<double> L, const SolveAr
 __global__ void __launch_bounds__(kNT) k_resid_init(Lvl<double> L, const double* __restrict__ x,
                                                     const double* __restrict__ b,
                                                     double* __restrict__ r, SolveState* st,
-                                                    double* part, cudaGraphConditionalHandle h,
+                                                    double* part, int again, cudaGraphConditionalHandle h,
                                                     int has_h) {
-  __shared__ double sh[kNT / 32];
+  __shared__ double sh[2 * kNT / 32];
   __shared__ int flag;
   double s_rr = 0.0, s_r0 = 0.0;
   // a zero iterate (no Dirichlet data, cold start) has r = r_0 = b: every product of the
@@ -180,29 +192,34 @@ __global__ void __launch_bounds__(kNT) k_resid_init(Lvl<double> L, const double*
     }
     if (r) r[k] = rv;
   }
-  const double a0 = block_sum<kNT>(s_rr, sh);
-  const double a1 = block_sum<kNT>(s_r0, sh);
+  double v[2] = {s_rr, s_r0};
+  block_sums<kNT, 2>(v, sh);
   if (threadIdx.x == 0) {
-    part[bid()] = a0;
-    part[nblocks() + bid()] = a1;
+    part[bid()] = v[0];
+    part[nblocks() + bid()] = v[1];
   }
   if (last_block_arrival(&st->ticket[0], nblocks(), &flag)) {
-    const double rr = reduce_partials<kNT>(part, nblocks(), sh);
-    const double q0 = reduce_partials<kNT>(part + nblocks(), nblocks(), sh);
+    reduce_partials<kNT, 2>(part, nblocks(), v, sh);
     if (threadIdx.x == 0) {
-      st->r0 = (q0 > 0.0) ? sqrt(q0) : 1.0;
-      decide(st, rr, h, has_h);
+      st->r0 = (v[1] > 0.0) ? sqrt(v[1]) : 1.0;
+      decide(st, v[0], h, has_h);
+      // the cycle and SOR loops record the residual before each iteration: the first one again
+      if (again && !st->done) {
+        if (st->hist_n < 256) st->hist[st->hist_n] = st->rel;
+        st->hist_n += 1;
+      }
     }
   }
 }
 
-// ||b - A x||^2 for the plain-cycle loop; optional r output; the last block decides.
+// Last kernel of a pass of the plain-cycle and SOR loops: ||b - A x||^2, optional r output; the last
+// block counts the iteration and decides.
 __global__ void __launch_bounds__(kNT) k_resid_check(Lvl<double> L, const double* __restrict__ x,
                                                      const double* __restrict__ b,
                                                      double* __restrict__ r, SolveState* st,
                                                      double* part, cudaGraphConditionalHandle h,
                                                      int has_h) {
-  __shared__ double sh[kNT / 32];
+  __shared__ double sh[2 * kNT / 32];
   __shared__ int flag;
   double s = 0.0;
   NODE_LOOP(L) {
@@ -214,11 +231,16 @@ __global__ void __launch_bounds__(kNT) k_resid_check(Lvl<double> L, const double
     }
     if (r) r[k] = rv;
   }
-  const double a0 = block_sum<kNT>(s, sh);
-  if (threadIdx.x == 0) part[bid()] = a0;
+  double v[1] = {s};
+  block_sums<kNT, 1>(v, sh);
+  if (threadIdx.x == 0) part[bid()] = v[0];
   if (last_block_arrival(&st->ticket[1], nblocks(), &flag)) {
-    const double rr = reduce_partials<kNT>(part, nblocks(), sh);
-    if (threadIdx.x == 0) decide(st, rr, h, has_h);
+    reduce_partials<kNT, 1>(part, nblocks(), v, sh);
+    if (threadIdx.x == 0) {
+      st->it += 1;
+      decide(st, v[0], h, 0);
+      end_of_pass(st, h, has_h);
+    }
   }
 }
 
@@ -246,22 +268,6 @@ __global__ void __launch_bounds__(kNT) k_add_f32(Lvl<double> L, double* __restri
   }
 }
 
-// Last node of every loop body: counts passes and ends the loop after 2 max_iters + 8
-// of them even if no convergence decision was reached (status: not converged).
-__global__ void k_loop_guard(SolveState* st, cudaGraphConditionalHandle h) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  st->guard += 1;
-  if (!st->done && st->guard > 2 * st->max_iters + 8) {
-    st->done = 1;
-    st->status = 6;
-    cudaGraphSetConditional(h, 0u);
-  }
-}
-
-__global__ void k_iter_inc(SolveState* st) {
-  if (!st->done && threadIdx.x == 0 && blockIdx.x == 0) st->it += 1;
-}
-
 // ---- flexible CG (FCG(1)): p = z + beta p_old, beta = -(z . q_old) / (p_old . q_old);
 // alpha = (p . r) / (p . q); x += alpha p; r -= alpha q.
 template <typename TZ>
@@ -272,7 +278,7 @@ __global__ void __launch_bounds__(kNT, kRedBlocksPerSM) k_fcg_zq(Lvl<double> L, 
     if (!st->done && bid() == 0 && threadIdx.x == 0) st->beta = 0.0;
     return;
   }
-  __shared__ double sh[kNT / 32];
+  __shared__ double sh[2 * kNT / 32];
   __shared__ int flag;
   const double is = (sizeof(TZ) == 4) ? st->inv_scale_r32 : 1.0;
   const bool f32ok = pow2_fits_f32(is);
@@ -292,13 +298,14 @@ __global__ void __launch_bounds__(kNT, kRedBlocksPerSM) k_fcg_zq(Lvl<double> L, 
             s += (sizeof(TZ) == 4 ? from_f32_scaled((float)zv[u], is, f32ok) : (double)zv[u]) * qv[u];
         });
   }
-  const double a0 = block_sum<kNT>(s, sh);
-  if (threadIdx.x == 0) part[bid()] = a0;
+  double v[1] = {s};
+  block_sums<kNT, 1>(v, sh);
+  if (threadIdx.x == 0) part[bid()] = v[0];
   if (last_block_arrival(&st->ticket[2], nblocks(), &flag)) {
-    const double zq = reduce_partials<kNT>(part, nblocks(), sh);
+    reduce_partials<kNT, 1>(part, nblocks(), v, sh);
     if (threadIdx.x == 0) {
-      st->zq = zq;
-      st->beta = (st->pq_old != 0.0) ? -zq / st->pq_old : 0.0;
+      st->zq = v[0];
+      st->beta = (st->pq_old != 0.0) ? -v[0] / st->pq_old : 0.0;
     }
   }
 }
@@ -312,7 +319,7 @@ __global__ void __launch_bounds__(kNT) k_fcg_pq(Lvl<double> L, const TZ* __restr
                                                 const double* __restrict__ r, SolveState* st,
                                                 double* part) {
   if (st->done) return;
-  __shared__ double sh[kNT / 32];
+  __shared__ double sh[2 * kNT / 32];
   __shared__ int flag;
   const double is = (sizeof(TZ) == 4) ? st->inv_scale_r32 : 1.0;
   const double beta = st->beta;
@@ -343,20 +350,19 @@ __global__ void __launch_bounds__(kNT) k_fcg_pq(Lvl<double> L, const TZ* __restr
     spq = fma(pn, qn, spq);
     spr = fma(pn, r[k], spr);
   }
-  const double a0 = block_sum<kNT>(spq, sh);
-  const double a1 = block_sum<kNT>(spr, sh);
+  double v[2] = {spq, spr};
+  block_sums<kNT, 2>(v, sh);
   if (threadIdx.x == 0) {
-    part[bid()] = a0;
-    part[nblocks() + bid()] = a1;
+    part[bid()] = v[0];
+    part[nblocks() + bid()] = v[1];
   }
   if (last_block_arrival(&st->ticket[3], nblocks(), &flag)) {
-    const double pq = reduce_partials<kNT>(part, nblocks(), sh);
-    const double pr = reduce_partials<kNT>(part + nblocks(), nblocks(), sh);
+    reduce_partials<kNT, 2>(part, nblocks(), v, sh);
     if (threadIdx.x == 0) {
-      st->pq = pq;
-      st->pr = pr;
-      st->alpha = (pq != 0.0) ? pr / pq : 0.0;
-      st->pq_old = pq;
+      st->pq = v[0];
+      st->pr = v[1];
+      st->alpha = (v[0] != 0.0) ? v[1] / v[0] : 0.0;
+      st->pq_old = v[0];
     }
   }
 }
@@ -393,7 +399,7 @@ __global__ void __launch_bounds__(kNT) k_fcg_q(Lvl<double> L, const double* __re
                                                double* __restrict__ q, SolveState* st,
                                                double* part) {
   if (st->done) return;
-  __shared__ double sh[kNT / 32];
+  __shared__ double sh[2 * kNT / 32];
   __shared__ int flag;
   double spq = 0.0, spr = 0.0;
   NODE_LOOP(L) {
@@ -404,20 +410,19 @@ __global__ void __launch_bounds__(kNT) k_fcg_q(Lvl<double> L, const double* __re
     spq = fma(p[k], qv, spq);
     spr = fma(p[k], r[k], spr);
   }
-  const double a0 = block_sum<kNT>(spq, sh);
-  const double a1 = block_sum<kNT>(spr, sh);
+  double v[2] = {spq, spr};
+  block_sums<kNT, 2>(v, sh);
   if (threadIdx.x == 0) {
-    part[bid()] = a0;
-    part[nblocks() + bid()] = a1;
+    part[bid()] = v[0];
+    part[nblocks() + bid()] = v[1];
   }
   if (last_block_arrival(&st->ticket[3], nblocks(), &flag)) {
-    const double pq = reduce_partials<kNT>(part, nblocks(), sh);
-    const double pr = reduce_partials<kNT>(part + nblocks(), nblocks(), sh);
+    reduce_partials<kNT, 2>(part, nblocks(), v, sh);
     if (threadIdx.x == 0) {
-      st->pq = pq;
-      st->pr = pr;
-      st->alpha = (pq != 0.0) ? pr / pq : 0.0;
-      st->pq_old = pq;
+      st->pq = v[0];
+      st->pr = v[1];
+      st->alpha = (v[0] != 0.0) ? v[1] / v[0] : 0.0;
+      st->pq_old = v[0];
     }
   }
 }
@@ -429,10 +434,9 @@ __global__ void __launch_bounds__(kNT) k_fcg_update(Lvl<double> L, double* __res
                                                     const double* __restrict__ p,
                                                     const double* __restrict__ q,
                                                     float* __restrict__ r32, int p32,
-                                                    SolveState* st, double* part,
-                                                    cudaGraphConditionalHandle h, int has_h) {
+                                                    SolveState* st, double* part) {
   if (st->done) return;
-  __shared__ double sh[kNT / 32];
+  __shared__ double sh[2 * kNT / 32];
   __shared__ int flag;
   const double alpha = st->alpha;
   const double sc = st->scale;
@@ -447,28 +451,33 @@ __global__ void __launch_bounds__(kNT) k_fcg_update(Lvl<double> L, double* __res
     if (r32) r32[(size_t)j * p32 + i] = to_f32_scaled(rv, sc, f32ok);
     s = fma(rv, rv, s);
   }
-  const double a0 = block_sum<kNT>(s, sh);
-  if (threadIdx.x == 0) part[bid()] = a0;
+  double v[1] = {s};
+  block_sums<kNT, 1>(v, sh);
+  if (threadIdx.x == 0) part[bid()] = v[0];
   if (last_block_arrival(&st->ticket[4], nblocks(), &flag)) {
-    const double rr = reduce_partials<kNT>(part, nblocks(), sh);
+    reduce_partials<kNT, 1>(part, nblocks(), v, sh);
     if (threadIdx.x == 0) {
       st->it += 1;
       if (r32) st->inv_scale_r32 = 1.0 / sc;
-      decide(st, rr, h, has_h, 1);
+      decide(st, v[0], 0, 0, 1);
     }
   }
 }
 
-// Residual replacement: when the recursive residual met rtol, r = b - A x is recomputed;
-// the solve stops only if the true residual meets rtol, else CG continues from it.
+// Last kernel of a CG pass; does nothing but close the pass unless the recursive residual met rtol.
+// Residual replacement: then r = b - A x is recomputed; the solve stops only if the true residual
+// meets rtol, else CG continues from it.
 __global__ void __launch_bounds__(kNT) k_fcg_verify(Lvl<double> L, const double* __restrict__ x,
                                                     const double* __restrict__ b,
                                                     double* __restrict__ r,
                                                     float* __restrict__ r32, int p32,
                                                     SolveState* st, double* part,
                                                     cudaGraphConditionalHandle h, int has_h) {
-  if (st->done || !st->verify) return;
-  __shared__ double sh[kNT / 32];
+  if (st->done || !st->verify) {
+    if (bid() == 0 && threadIdx.x == 0) end_of_pass(st, h, has_h);
+    return;
+  }
+  __shared__ double sh[2 * kNT / 32];
   __shared__ int flag;
   const double sc = st->scale;
   const bool f32ok = pow2_fits_f32(sc);
@@ -483,21 +492,22 @@ __global__ void __launch_bounds__(kNT) k_fcg_verify(Lvl<double> L, const double*
     r[k] = rv;
     if (r32) r32[(size_t)j * p32 + i] = to_f32_scaled(rv, sc, f32ok);
   }
-  const double a0 = block_sum<kNT>(s, sh);
-  if (threadIdx.x == 0) part[bid()] = a0;
+  double v[1] = {s};
+  block_sums<kNT, 1>(v, sh);
+  if (threadIdx.x == 0) part[bid()] = v[0];
   if (last_block_arrival(&st->ticket[5], nblocks(), &flag)) {
-    const double rr = reduce_partials<kNT>(part, nblocks(), sh);
+    reduce_partials<kNT, 1>(part, nblocks(), v, sh);
     if (threadIdx.x == 0) {
       st->verify = 0;
       if (r32) st->inv_scale_r32 = 1.0 / sc;
-      decide(st, rr, h, has_h, 0);
+      decide(st, v[0], h, 0, 0);
       // the recursive residual keeps meeting rtol but the true one does not: the true
       // residual has reached its rounding floor above rtol; stop (not converged)
       if (!st->done && ++st->verify_fail >= kMaxVerifyFail) {
         st->done = 1;
         st->status = 6;
-        if (has_h) cudaGraphSetConditional(h, 0u);
       }
+      end_of_pass(st, h, has_h);
     }
   }
 }
@@ -546,10 +556,10 @@ cudaError_t launch_solve_init(const OpF64& A, const SolveArgs* a, const double* 
   CHK();
 }
 cudaError_t launch_resid_init(const OpF64& A, const double* x, const double* b, double* r,
-                              SolveState* st, double* part, cudaGraphConditionalHandle h,
+                              SolveState* st, double* part, int again, cudaGraphConditionalHandle h,
                               int has_h, cudaStream_t s) {
   const Lvl<double> L = lvl_of(A);
-  k_resid_init<<<red_grid(L.nx, L.nyr), kNT, 0, s>>>(L, x, b, r, st, part, h, has_h);
+  k_resid_init<<<red_grid(L.nx, L.nyr), kNT, 0, s>>>(L, x, b, r, st, part, again, h, has_h);
   CHK();
 }
 cudaError_t launch_resid_check(const OpF64& A, const double* x, const double* b, double* r,
@@ -569,14 +579,6 @@ cudaError_t launch_add_f32(const OpF64& A, double* x, const float* e32, int pitc
                            SolveState* st, cudaStream_t s) {
   const Lvl<double> L = lvl_of(A);
   k_add_f32<<<red_grid(L.nx, L.nyr), kNT, 0, s>>>(L, x, e32, pitch32, st);
-  CHK();
-}
-cudaError_t launch_loop_guard(SolveState* st, cudaGraphConditionalHandle h, cudaStream_t s) {
-  k_loop_guard<<<1, 32, 0, s>>>(st, h);
-  CHK();
-}
-cudaError_t launch_iter_inc(SolveState* st, cudaStream_t s) {
-  k_iter_inc<<<1, 32, 0, s>>>(st);
   CHK();
 }
 template <typename TZ>
@@ -609,9 +611,9 @@ cudaError_t launch_fcg_pq<float>(const OpF64& A, const float* z, int zp, double*
 }
 cudaError_t launch_fcg_update(const OpF64& A, double* x, double* r, const double* p,
                               const double* q, float* r32, int p32, SolveState* st, double* part,
-                              cudaGraphConditionalHandle h, int has_h, cudaStream_t s) {
+                              cudaStream_t s) {
   const Lvl<double> L = lvl_of(A);
-  k_fcg_update<<<red_grid(L.nx, L.nyr), kNT, 0, s>>>(L, x, r, p, q, r32, p32, st, part, h, has_h);
+  k_fcg_update<<<red_grid(L.nx, L.nyr), kNT, 0, s>>>(L, x, r, p, q, r32, p32, st, part);
   CHK();
 }
 cudaError_t launch_fcg_verify(const OpF64& A, const double* x, const double* b, double* r,

@@ -93,47 +93,69 @@ struct SolveState {
 static_assert(sizeof(SolveState) % 8 == 0, "SolveState is copied as 8-byte words");
 
 // ---- deterministic block reduction -------------------------------------------------
-// Sums v over the block in a fixed order (warp shuffle tree, then warps in order).
-template <int NT>
-__device__ __forceinline__ double block_sum(double v, double* sh /* >= NT/32 */) {
+// Sums each of the K values of v over the block in a fixed order (warp shuffle tree, then warps in
+// order, one lane per value); valid in thread 0.
+template <int NT, int K>
+__device__ __forceinline__ void block_sums(double (&v)[K], double* sh /* >= K NT/32 */) {
+  constexpr int NW = NT / 32;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < K; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) sh[warp] = v;
+  if (lane == 0)
+#pragma unroll
+    for (int q = 0; q < K; ++q) sh[q * NW + warp] = v[q];
   __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0) {
-    for (int w = 0; w < NT / 32; ++w) t += sh[w];
+  if (warp == 0) {
+    double t = 0.0;
+    if (lane < K) {
+#pragma unroll
+      for (int w = 0; w < NW; ++w) t += sh[lane * NW + w];
+    }
+#pragma unroll
+    for (int q = 0; q < K; ++q) v[q] = __shfl_sync(0xffffffffu, t, q);
   }
   __syncthreads();
-  return t;  // valid in thread 0
 }
 
-// After each block has written partial[blockLinear], the block that arrives last
+// After thread 0 of each block has written the block's partial sums, the block that arrives last
 // (counted with an atomic ticket) returns true in all its threads; it then owns the
 // final fixed-order reduction.  The ticket is reset for the next use.
 __device__ __forceinline__ bool last_block_arrival(unsigned int* ticket, unsigned int nblocks,
                                                    int* sh_flag) {
-  __threadfence();
-  __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned int t = atomicAdd(ticket, 1u);
+    __threadfence();  // the partial sums (written by this thread) before the ticket
+    const unsigned int t = atomicAdd(ticket, 1u);
     *sh_flag = (t == nblocks - 1);
+    if (t == nblocks - 1) *ticket = 0u;
+    __threadfence();
   }
   __syncthreads();
-  bool last = *sh_flag;
-  if (last && threadIdx.x == 0) *ticket = 0u;
-  if (last) __threadfence();
-  return last;
+  return *sh_flag;
 }
 
-// Fixed-order sum of n partials by one block (tree over a strided split; the order
-// depends only on n and the block size).
-template <int NT>
-__device__ double reduce_partials(const double* __restrict__ part, int n, double* sh) {
-  double v = 0.0;
-  for (int k = threadIdx.x; k < n; k += NT) v += ((volatile const double*)part)[k];
-  return block_sum<NT>(v, sh);
+// Fixed-order sums of K rows of n partials (row q at part + q n) by one block (tree over a strided
+// split; the order depends only on n and the block size); valid in thread 0.  A thread's loads are
+// issued together: one at a time, each waits a round trip to L2.
+template <int NT, int K>
+__device__ __forceinline__ void reduce_partials(const double* part, int n, double (&v)[K], double* sh) {
+  constexpr int B = 8;
+#pragma unroll
+  for (int q = 0; q < K; ++q) v[q] = 0.0;
+  for (int k0 = threadIdx.x; k0 < n; k0 += B * NT) {
+    double w[K][B];
+#pragma unroll
+    for (int q = 0; q < K; ++q)
+#pragma unroll
+      for (int u = 0; u < B; ++u) w[q][u] = k0 + u * NT < n ? __ldcg(part + (size_t)q * n + k0 + u * NT) : 0.0;
+#pragma unroll
+    for (int q = 0; q < K; ++q)
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (k0 + u * NT < n) v[q] += w[q][u];
+  }
+  block_sums<NT, K>(v, sh);
 }
 
 }  // namespace mg

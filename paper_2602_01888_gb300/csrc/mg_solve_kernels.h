@@ -30,7 +30,7 @@ dim3 red_grid(int nx, int nyr);
 cudaError_t launch_solve_init(const OpF64& A, const SolveArgs* a, const double* D, double* x,
                               double* b, SolveState* st, cudaStream_t s);
 cudaError_t launch_resid_init(const OpF64& A, const double* x, const double* b, double* r,
-                              SolveState* st, double* part, cudaGraphConditionalHandle h,
+                              SolveState* st, double* part, int again, cudaGraphConditionalHandle h,
                               int has_h, cudaStream_t s);
 cudaError_t launch_resid_check(const OpF64& A, const double* x, const double* b, double* r,
                                SolveState* st, double* part, cudaGraphConditionalHandle h,
@@ -39,8 +39,6 @@ cudaError_t launch_r_to_f32(const OpF64& A, const double* r, float* b32, int pit
                             SolveState* st, cudaStream_t s);
 cudaError_t launch_add_f32(const OpF64& A, double* x, const float* e32, int pitch32,
                            SolveState* st, cudaStream_t s);
-cudaError_t launch_iter_inc(SolveState* st, cudaStream_t s);
-cudaError_t launch_loop_guard(SolveState* st, cudaGraphConditionalHandle h, cudaStream_t s);
 template <typename TZ>
 cudaError_t launch_fcg_zq(const OpF64& A, const TZ* z, int zp, const double* q, SolveState* st,
                           double* part, cudaStream_t s);
@@ -49,7 +47,7 @@ cudaError_t launch_fcg_pq(const OpF64& A, const TZ* z, int zp, double* p, double
                           SolveState* st, double* part, cudaStream_t s);
 cudaError_t launch_fcg_update(const OpF64& A, double* x, double* r, const double* p,
                               const double* q, float* r32, int p32, SolveState* st, double* part,
-                              cudaGraphConditionalHandle h, int has_h, cudaStream_t s);
+                              cudaStream_t s);
 cudaError_t launch_fcg_verify(const OpF64& A, const double* x, const double* b, double* r,
                               float* r32, int p32, SolveState* st, double* part,
                               cudaGraphConditionalHandle h, int has_h, cudaStream_t s);

@@ -775,7 +775,8 @@ static mg_status emit_vcycle_on(mg_problem* P, T* x0, T* b0, const mg_solve_opts
   return MG_OK;
 }
 
-// Body of one outer iteration.
+// One pass of the solve loop: an outer iteration and, in its last kernel, the decision whether
+// another follows (nothing of a pass is launched after convergence).
 static mg_status emit_body(mg_problem* P, const mg_solve_opts& o, cudaGraphConditionalHandle h,
                            int has_h, cudaStream_t s) {
   LevelMem& F = P->lev[0];
@@ -784,31 +785,27 @@ static mg_status emit_body(mg_problem* P, const mg_solve_opts& o, cudaGraphCondi
   const bool mixed = (o.precision == MG_PREC_MIXED);
   mg_status st;
   if (o.outer == MG_OUTER_SOR) {  // single-level baseline: nu1 SOR sweeps per tested iteration
-    CU(launch_resid_check(F.A, F.x, F.b, nullptr, P->st, P->part, h, has_h, s));
     CU(launch_sor<double>(F.A, F.x, F.b, o.nu1, o.omega_j, skip, s));
-    CU(launch_iter_inc(P->st, s));
+    CU(launch_resid_check(F.A, F.x, F.b, nullptr, P->st, P->part, h, has_h, s));
     return MG_OK;
   }
   if (o.outer == MG_OUTER_VCYCLE) {
     if (!mixed) {
-      CU(launch_resid_check(F.A, F.x, F.b, nullptr, P->st, P->part, h, has_h, s));
       double* res = nullptr;
       if ((st = emit_vcycle_on<double>(P, F.x, F.b, o, skip, s, &res))) return st;
       if (res != F.x) CU(cudaMemcpyAsync(F.x, res, n0 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+      CU(launch_resid_check(F.A, F.x, F.b, nullptr, P->st, P->part, h, has_h, s));
     } else {
-      CU(launch_resid_check(F.A, F.x, F.b, P->r, P->st, P->part, h, has_h, s));
       CU(launch_r_to_f32(F.A, P->r, F.b32, F.A32.pitch, P->st, s));
       float* res = nullptr;
       if ((st = emit_vcycle_on<float>(P, F.x32, F.b32, o, skip, s, &res, true))) return st;
       CU(launch_add_f32(F.A, F.x, res, F.A32.pitch, P->st, s));
+      CU(launch_resid_check(F.A, F.x, F.b, P->r, P->st, P->part, h, has_h, s));
     }
-    CU(launch_iter_inc(P->st, s));
     return MG_OK;
   }
   // flexible CG preconditioned by one V-cycle; for the mixed path the cycle's right-hand
   // side r32 was written by the previous update (or the initialisation / verification)
-  CU(launch_fcg_verify(F.A, F.x, F.b, P->r, mixed ? F.b32 : nullptr, F.A32.pitch, P->st, P->part, h,
-                       has_h, s));
   if (!mixed) {
     double* res = nullptr;
     if ((st = emit_vcycle_on<double>(P, P->z, P->r, o, skip, s, &res, true))) return st;
@@ -820,9 +817,21 @@ static mg_status emit_body(mg_problem* P, const mg_solve_opts& o, cudaGraphCondi
     CU(launch_fcg_zq<float>(F.A, res, F.A32.pitch, P->q, P->st, P->part, s));
     CU(launch_fcg_pq<float>(F.A, res, F.A32.pitch, P->p, P->q, P->r, P->st, P->part, s));
   }
-  CU(launch_fcg_update(F.A, F.x, P->r, P->p, P->q, mixed ? F.b32 : nullptr, F.A32.pitch, P->st,
-                       P->part, h, has_h, s));
+  CU(launch_fcg_update(F.A, F.x, P->r, P->p, P->q, mixed ? F.b32 : nullptr, F.A32.pitch, P->st, P->part, s));
+  CU(launch_fcg_verify(F.A, F.x, F.b, P->r, mixed ? F.b32 : nullptr, F.A32.pitch, P->st, P->part, h,
+                       has_h, s));
   return MG_OK;
+}
+
+// The residual of the initial iterate and the decision whether to iterate at all; r is kept where
+// the loop starts from it (CG, and the FP32 cycle's right-hand side).
+static cudaError_t emit_initial_residual(mg_problem* P, const mg_solve_opts& o, cudaGraphConditionalHandle h, int has_h,
+                                         cudaStream_t s) {
+  LevelMem& F = P->lev[0];
+  const bool fcg = o.outer == MG_OUTER_FCG, mixed = o.precision == MG_PREC_MIXED;
+  cudaError_t e = launch_resid_init(F.A, F.x, F.b, fcg || mixed ? P->r : nullptr, P->st, P->part, fcg ? 0 : 1, h, has_h, s);
+  if (!e && fcg && mixed) e = launch_r_to_f32(F.A, P->r, F.b32, F.A32.pitch, P->st, s);
+  return e;
 }
 
 uint64_t graph_key(const mg_solve_opts& o) {
@@ -837,15 +846,14 @@ uint64_t graph_key(const mg_solve_opts& o) {
 }
 
 // One solve captured into the graph g that stream cs is capturing: init -> initial
-// residual (sets the condition) -> WHILE(condition){ one outer iteration; the last kernel
-// re-sets the condition } -> copy out.  `args` is the device argument block the kernels
+// residual (sets the condition) -> WHILE(condition){ one outer iteration; its last kernel
+// decides and re-sets the condition } -> copy out.  `args` is the device argument block the kernels
 // read; the loop body is captured on cs2.  Counts the kernel nodes it adds.
 static mg_status capture_solve_chain(mg_problem* P, const mg_solve_opts& o, SolveArgs* args,
                                      cudaStream_t cs, cudaStream_t cs2, cudaGraph_t g,
                                      int* fixed_kernels, int* body_kernels) {
   LevelMem& F = P->lev[0];
-  const bool fcg = (o.outer == MG_OUTER_FCG);
-  const bool r32 = fcg && o.precision == MG_PREC_MIXED;
+  const bool r32 = o.outer == MG_OUTER_FCG && o.precision == MG_PREC_MIXED;
   cudaStreamCaptureStatus cst;
   const cudaGraphNode_t* deps = nullptr;
   size_t ndeps = 0;
@@ -853,9 +861,7 @@ static mg_status capture_solve_chain(mg_problem* P, const mg_solve_opts& o, Solv
   if (cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault) != cudaSuccess)
     return set_error(MG_ERR_CUDA, "conditional handle creation failed");
   if (launch_solve_init(F.A, args, P->D, F.x, F.b, P->st, cs) != cudaSuccess ||
-      launch_resid_init(F.A, F.x, F.b, fcg ? P->r : nullptr, P->st, P->part, h, 1, cs) !=
-          cudaSuccess ||
-      (r32 && launch_r_to_f32(F.A, P->r, F.b32, F.A32.pitch, P->st, cs) != cudaSuccess))
+      emit_initial_residual(P, o, h, 1, cs) != cudaSuccess)
     return set_error(MG_ERR_CUDA, "capture of solve init failed");
   *fixed_kernels = 3 + (r32 ? 1 : 0);
   if (cudaStreamGetCaptureInfo(cs, &cst, nullptr, nullptr, &deps, nullptr, &ndeps) != cudaSuccess)
@@ -876,8 +882,6 @@ static mg_status capture_solve_chain(mg_problem* P, const mg_solve_opts& o, Solv
       cudaSuccess)
     return set_error(MG_ERR_CUDA, "body capture failed to start");
   mg_status st = emit_body(P, o, h, 1, cs2);
-  if (!st && launch_loop_guard(P->st, h, cs2) != cudaSuccess)
-    st = set_error(MG_ERR_CUDA, "capture of the loop guard failed");
   cudaGraph_t body_out = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(cs2, &body_out);
   if (!st && e2 != cudaSuccess)
@@ -1046,11 +1050,8 @@ static bool host_loop_mode() {
 
 static mg_status run_host_loop(mg_problem* P, const mg_solve_opts& o, cudaStream_t s, int* passes) {
   LevelMem& F = P->lev[0];
-  const bool fcg = (o.outer == MG_OUTER_FCG);
   CU(launch_solve_init(F.A, P->args, P->D, F.x, F.b, P->st, s));
-  CU(launch_resid_init(F.A, F.x, F.b, fcg ? P->r : nullptr, P->st, P->part, 0, 0, s));
-  if (fcg && o.precision == MG_PREC_MIXED)
-    CU(launch_r_to_f32(F.A, P->r, F.b32, F.A32.pitch, P->st, s));
+  CU(emit_initial_residual(P, o, 0, 0, s));
   *passes = 0;
   for (int pass = 0; pass < 2 * o.max_iters + 8; ++pass) {
     int done = 0;
@@ -1098,8 +1099,7 @@ mg_status enqueue_solve(mg_problem* P, const mg_solve_opts& o, const double* rho
     int passes = 0;
     mg_status st = run_host_loop(P, o, s, &passes);
     if (st) return st;
-    // the graph's loop body also holds the loop guard, which the host loop replaces
-    P->last_fixed_kernels = it->second.fixed_kernels + passes * (it->second.body_kernels - 1);
+    P->last_fixed_kernels = it->second.fixed_kernels + passes * it->second.body_kernels;
     P->last_body_kernels = 0;
   } else {
     CU(cudaGraphLaunch(it->second.exec, s));
