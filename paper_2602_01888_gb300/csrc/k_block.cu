@@ -25,8 +25,9 @@
 // host): 129^2 15.5 -> 5.3 us, 513^2 14.4 -> 6.2 us, 1025^2 36.9 -> 16.7 us (tile kernels), 4097^2
 // 203 -> 164 us (row marching).  Marching a strip with everything in one warp's registers, without
 // any barrier, was slower (177 us at 4097^2, 18 us at 1025^2: two warps a scheduler cannot hide the
-// chain of a step).  FP64 is not chosen by the size rule: its phases wait on the FP64 pipe's latency
-// (1025^2: 41 us a sweep against 33 us for the per-colour kernels).
+// chain of a step).  FP64 (32 x 32 regions, two CTAs an SM) is bound by a phase's chain of ten FP64
+// operations: two sweeps with the restriction or the correction take about 12 us at 65^2 and 129^2,
+// where the fused tile kernel took 18 us without either.
 //
 // Operations per node and their order are those of the per-colour kernels and of
 // k_resid_restrict, so the results are the same bit for bit.
@@ -39,18 +40,19 @@
 
 namespace mg {
 
-template <typename T, int NS, int TY, bool RR>
+template <typename T, int NS, int TX_, int TY, bool RR>
 struct BlockGeom {
-  static constexpr int TX = 32;                      // blocks a row (one warp)
+  static constexpr int TX = TX_;                     // blocks a row (a warp or half a warp)
   static constexpr int RX = 2 * TX, RY = 2 * TY;     // nodes of the staged region
   static constexpr int VEC = 16 / (int)sizeof(T);    // elements of a 16-byte chunk
   // halo columns (left, right) and rows (below, above): see the reach in the head of this file; left
   // and below rounded up to whole chunks and blocks, the owned width to whole chunks
-  static constexpr int HL = NS == 2 ? 8 : (RR ? (VEC == 4 ? 8 : 6) : 4);
-  static constexpr int HR = NS == 2 ? (RR ? 8 : 4) : (RR || VEC == 4 ? 4 : 2);
+  static constexpr int HL = VEC == 4 ? (NS == 2 || RR ? 8 : 4) : (NS == 2 ? (RR ? 8 : 6) : (RR ? 6 : 4));
+  static constexpr int HR = VEC == 4 ? (NS == 2 && RR ? 8 : 4) : (NS == 2 ? (RR ? 6 : 4) : (RR ? 4 : 2));
   static constexpr int HB = 4 * NS + (RR ? 2 : 0), HT = 4 * NS;
   static constexpr int OX = RX - HL - HR, OY = RY - HB - HT;
   static constexpr int THREADS = TX * TY;
+  static constexpr int CTAS = sizeof(T) == 8 ? 2 : 1;  // resident CTAs a SM
   static constexpr int PLANE = TX * TY;
   static constexpr int CHX = RX / VEC, CHUNKS = CHX * RY;  // chunks of a row, of an array
   static constexpr int CW = TX + 1, CH = TY + 1;     // coarse nodes under the region
@@ -61,7 +63,7 @@ struct BlockGeom {
   static constexpr int SMEM = ((ELEMS * (int)sizeof(T) + 15) / 16) * 16;
   static_assert(OX > 0 && OY > 0, "no owned nodes");
   static_assert(HL % VEC == 0 && OX % VEC == 0 && OX % 2 == 0 && OY % 2 == 0, "region starts on a chunk and a block");
-  static_assert(SMEM <= 227 * 1024, "must fit in shared memory");
+  static_assert(CTAS * (SMEM + 1024 + 32) <= 228 * 1024, "resident CTAs must fit in shared memory");
 };
 
 template <int BYTES>
@@ -85,13 +87,13 @@ struct T2<double> {
   using type = double2;
 };
 
-template <typename T, int NS, int TY, bool REV, bool RR, bool FIVE>
-__global__ void __launch_bounds__(32 * TY, 1)
+template <typename T, int NS, int TX, int TY, bool REV, bool RR, bool FIVE>
+__global__ void __launch_bounds__(TX * TY, BlockGeom<T, NS, TX, TY, RR>::CTAS)
     k_smooth_block(Lvl<T> L, const T* __restrict__ xin, T* __restrict__ xout, const T* __restrict__ b,
                    const T* __restrict__ eH, T* __restrict__ bH, int pitchc, int nxc, int nyc, int nyrc, int tiles_x,
                    int ntiles, const int* __restrict__ skip) {
   if (skip && *skip) return;
-  using G = BlockGeom<T, NS, TY, RR>;
+  using G = BlockGeom<T, NS, TX, TY, RR>;
   using P2 = typename T2<T>::type;
   constexpr int RX = G::RX, RY = G::RY, PL = G::PLANE, ARR = G::ARR;
   extern __shared__ __align__(16) unsigned char blk_smem[];
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
   T* const es = plane + 4 * PL;
   T* const dg = es + ((G::CW * G::CH + 3) & ~3);  // 2 x ARR (RR)
   T* const rp = dg + 2 * ARR;                     // residual planes b, c, d (RR)
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, t = threadIdx.x;
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX, t = threadIdx.x;
   const int p = L.pitch;
 
   auto request = [&](int tile, int buf) {
@@ -188,7 +190,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
       if (mc) xc += T(0.5) * (ea + ec);
       if (md) xd += T(0.25) * ((ea + eb) + (ec + ed));
     }
-    T* const A = plane + ty * 32 + tx;
+    T* const A = plane + ty * TX + tx;
     T* const B = A + PL;
     T* const C = B + PL;
     T* const D = C + PL;
@@ -205,12 +207,12 @@ __global__ void __launch_bounds__(32 * TY, 1)
       T s = E0.x * xb;
       s = fma(E0l, B[-1], s);
       s = fma(N0.x, xc, s);
-      s = fma(Nm.x, C[-32], s);
+      s = fma(Nm.x, C[-TX], s);
       if (!FIVE) {
         s = fma(NE0.x, xd, s);
-        s = fma(NEml, D[-33], s);
+        s = fma(NEml, D[-TX - 1], s);
         s = fma(NW0.x, D[-1], s);
-        s = fma(NWm.y, D[-32], s);
+        s = fma(NWm.y, D[-TX], s);
       }
       return s;
     };
@@ -218,24 +220,24 @@ __global__ void __launch_bounds__(32 * TY, 1)
       T s = E0.y * A[1];
       s = fma(E0.x, xa, s);
       s = fma(N0.y, xd, s);
-      s = fma(Nm.y, D[-32], s);
+      s = fma(Nm.y, D[-TX], s);
       if (!FIVE) {
         s = fma(NE0.y, C[1], s);
-        s = fma(NEm.x, C[-32], s);
+        s = fma(NEm.x, C[-TX], s);
         s = fma(NW0.y, xc, s);
-        s = fma(NWmr, C[-31], s);
+        s = fma(NWmr, C[-TX + 1], s);
       }
       return s;
     };
     auto sum_c = [&]() {
       T s = E1.x * xd;
       s = fma(E1l, D[-1], s);
-      s = fma(N1.x, A[32], s);
+      s = fma(N1.x, A[TX], s);
       s = fma(N0.x, xa, s);
       if (!FIVE) {
-        s = fma(NE1.x, B[32], s);
+        s = fma(NE1.x, B[TX], s);
         s = fma(NE0l, B[-1], s);
-        s = fma(NW1.x, B[31], s);
+        s = fma(NW1.x, B[TX - 1], s);
         s = fma(NW0.y, xb, s);
       }
       return s;
@@ -243,12 +245,12 @@ __global__ void __launch_bounds__(32 * TY, 1)
     auto sum_d = [&]() {
       T s = E1.y * C[1];
       s = fma(E1.x, xc, s);
-      s = fma(N1.y, B[32], s);
+      s = fma(N1.y, B[TX], s);
       s = fma(N0.y, xb, s);
       if (!FIVE) {
-        s = fma(NE1.y, A[33], s);
+        s = fma(NE1.y, A[TX + 1], s);
         s = fma(NE0.x, xa, s);
-        s = fma(NW1.y, A[32], s);
+        s = fma(NW1.y, A[TX], s);
         s = fma(NW0r, A[1], s);
       }
       return s;
@@ -297,7 +299,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
       const T rb = mb ? b0.y - fma(g0.y, xb, sum_b()) : T(0);
       const T rc = mc ? b1.x - fma(g1.x, xc, sum_c()) : T(0);
       const T rd = md ? b1.y - fma(g1.y, xd, sum_d()) : T(0);
-      T* const Rb = rp + ty * 32 + tx;
+      T* const Rb = rp + ty * TX + tx;
       T* const Rc = Rb + PL;
       T* const Rd = Rc + PL;
       *Rb = rb;
@@ -309,8 +311,8 @@ __global__ void __launch_bounds__(32 * TY, 1)
         const bool unk = (I >= 1 && I <= nxc - 2) && (L.periodic || (J >= 1 && J <= nyc - 2));
         T v = T(0);
         if (unk) {
-          const T edge = Rb[-1] + rb + Rc[-32] + rc;
-          const T corner = Rd[-33] + Rd[-32] + Rd[-1] + rd;
+          const T edge = Rb[-1] + rb + Rc[-TX] + rc;
+          const T corner = Rd[-TX - 1] + Rd[-TX] + Rd[-1] + rd;
           v = (T(4) * ra + T(2) * edge + corner) * T(0.0625);
         }
         bH[(size_t)J * pitchc + I] = v;
@@ -337,19 +339,19 @@ bool block_can(const Op<T>& A, const T* xin, const T* xout, const T* b) {
   return A.pitch % (16 / (int)sizeof(T)) == 0 && all % 16 == 0 && !(A.periodic && (A.ny - 1) % 2);
 }
 
-template <typename T, int NS, int TY, bool RR>
+template <typename T, int NS, int TX, int TY, bool RR>
 static cudaError_t block_impl(const Op<T>& A, const T* xin, T* xout, const T* b, int rev, const T* eH, T* bH,
                               int pitch_c, const int* skip, cudaStream_t s) {
-  using G = BlockGeom<T, NS, TY, RR>;
+  using G = BlockGeom<T, NS, TX, TY, RR>;
   auto raise = [](auto kern) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM + 32);
   };
   static const cudaError_t attr = [&] {
-    cudaError_t e = raise(k_smooth_block<T, NS, TY, false, RR, false>);
-    if (!e) e = raise(k_smooth_block<T, NS, TY, false, RR, true>);
+    cudaError_t e = raise(k_smooth_block<T, NS, TX, TY, false, RR, false>);
+    if (!e) e = raise(k_smooth_block<T, NS, TX, TY, false, RR, true>);
     if constexpr (!RR) {
-      if (!e) e = raise(k_smooth_block<T, NS, TY, true, RR, false>);
-      if (!e) e = raise(k_smooth_block<T, NS, TY, true, RR, true>);
+      if (!e) e = raise(k_smooth_block<T, NS, TX, TY, true, RR, false>);
+      if (!e) e = raise(k_smooth_block<T, NS, TX, TY, true, RR, true>);
     }
     return e;
   }();
@@ -357,16 +359,16 @@ static cudaError_t block_impl(const Op<T>& A, const T* xin, T* xout, const T* b,
   const Lvl<T> L = lvl_of(A);
   const int nxc = (A.nx - 1) / 2 + 1, nyc = (A.ny - 1) / 2 + 1, nyrc = rows_stored(nyc, A.periodic);
   const int tx = (L.nx + G::OX - 1) / G::OX, ty = (L.nyr + G::OY - 1) / G::OY, ntiles = tx * ty;
-  const int grid = ntiles < blk_sms() ? ntiles : blk_sms();
+  const int slots = blk_sms() * G::CTAS, grid = ntiles < slots ? ntiles : slots;
   auto go = [&](auto kern) {
     kern<<<grid, G::THREADS, G::SMEM + 32, s>>>(L, xin, xout, b, eH, bH, pitch_c, nxc, nyc, nyrc, tx, ntiles, skip);
     return cudaGetLastError();
   };
   if constexpr (!RR) {
     if (rev)
-      return L.five_point ? go(k_smooth_block<T, NS, TY, true, RR, true>) : go(k_smooth_block<T, NS, TY, true, RR, false>);
+      return L.five_point ? go(k_smooth_block<T, NS, TX, TY, true, RR, true>) : go(k_smooth_block<T, NS, TX, TY, true, RR, false>);
   }
-  return L.five_point ? go(k_smooth_block<T, NS, TY, false, RR, true>) : go(k_smooth_block<T, NS, TY, false, RR, false>);
+  return L.five_point ? go(k_smooth_block<T, NS, TX, TY, false, RR, true>) : go(k_smooth_block<T, NS, TX, TY, false, RR, false>);
 }
 
 template <typename T>
@@ -374,27 +376,26 @@ cudaError_t launch_smooth_block(const Op<T>& A, const T* xin, T* xout, const T* 
                                 int pitch_c, const int* skip, cudaStream_t s) {
   if (xin == xout || !block_can(A, xin, xout, b) || (bH && (rev || eH || (A.nx - 1) % 2 || (A.ny - 1) % 2)))
     return cudaErrorInvalidValue;
+  if (ns != 1 && ns != 2) return cudaErrorInvalidValue;
   const int nyr = rows_stored(A.ny, A.periodic);
+  auto go = [&](auto ns_c, auto tx_c, auto ty_c) {
+    constexpr int NS = decltype(ns_c)::value, TX = decltype(tx_c)::value, TY = decltype(ty_c)::value;
+    return bH ? block_impl<T, NS, TX, TY, true>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s)
+              : block_impl<T, NS, TX, TY, false>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s);
+  };
+  using One = std::integral_constant<int, 1>;
+  using Two = std::integral_constant<int, 2>;
+  using N16 = std::integral_constant<int, 16>;
+  using N32 = std::integral_constant<int, 32>;
   if constexpr (sizeof(T) == 4) {
     // tall tiles (64 rows) where they fill the GPU, half as tall ones on small levels
     const bool tall = (long long)A.nx * nyr > 48LL * 16 * 152;
-    if (ns == 2) {
-      if (bH)
-        return tall ? block_impl<T, 2, 32, true>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s)
-                    : block_impl<T, 2, 16, true>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s);
-      return tall ? block_impl<T, 2, 32, false>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s)
-                  : block_impl<T, 2, 16, false>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s);
-    }
-    if (ns != 1) return cudaErrorInvalidValue;
-    if (bH)
-      return tall ? block_impl<T, 1, 32, true>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s)
-                  : block_impl<T, 1, 16, true>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s);
-    return tall ? block_impl<T, 1, 32, false>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s)
-                : block_impl<T, 1, 16, false>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s);
+    if (ns == 2) return tall ? go(Two(), N32(), N32()) : go(Two(), N32(), N16());
+    return tall ? go(One(), N32(), N32()) : go(One(), N32(), N16());
   } else {
-    if (ns != 1) return cudaErrorInvalidValue;
-    if (bH) return block_impl<T, 1, 16, true>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s);
-    return block_impl<T, 1, 16, false>(A, xin, xout, b, rev, eH, bH, pitch_c, skip, s);
+    // 32 x 32 regions: a phase is a chain of ten FP64 operations whatever the tile, so small tiles on
+    // many SMs (the levels this kernel is chosen for have few)
+    return ns == 2 ? go(Two(), N16(), N16()) : go(One(), N16(), N16());
   }
 }
 

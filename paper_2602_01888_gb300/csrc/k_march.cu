@@ -561,11 +561,11 @@ __global__ void __launch_bounds__(MarchGeom<T, CFG>::THREADS, MarchGeom<T, CFG>:
   }
 }
 
-// Variants: kMarchCfg gives the configuration of MarchGeom, or -ns for a register-block pass of ns
+// Variants: kMarchCfg gives the configuration of MarchGeom, or -2 for a register-block pass of two
 // sweeps (k_block.cu).  Variant 0 is each precision's default: FP32 the register blocks, FP64
 // configuration 3.
 constexpr int kMarchCfgF32[] = {-2, 0, 1, 2, 3, 4};
-constexpr int kMarchCfgF64[] = {3, 1, 2, 0, -1};
+constexpr int kMarchCfgF64[] = {3, 1, 2, 0, -2};
 
 template <typename T>
 int march_variants() {
@@ -591,7 +591,7 @@ static SmoothVariant march_cfg() {
 template <typename T>
 SmoothVariant march_variant(int v) {
   const int cfg = march_cfg_of<T>(v);
-  if (cfg < 0) return {block_tile_width<T>(-cfg), 0, -cfg};
+  if (cfg < 0) return {block_tile_width<T>(), 0, -cfg};
   if constexpr (sizeof(T) == 8) {
     switch (cfg) {
       case 1: return march_cfg<double, 1>();

@@ -6,15 +6,10 @@
 
 namespace mg {
 
-// Sweeps of one pass: FP32 two (or one), FP64 one.
+// Owned columns of a tile of two sweeps a pass, without the residual.
 template <typename T>
-constexpr int block_sweeps() {
-  return sizeof(T) == 4 ? 2 : 1;
-}
-// Owned columns of a tile without the residual.
-template <typename T>
-constexpr int block_tile_width(int ns) {
-  return ns == 2 ? 52 : (sizeof(T) == 4 ? 56 : 58);
+constexpr int block_tile_width() {
+  return sizeof(T) == 4 ? 52 : 22;
 }
 
 // Whether the kernel can run on these arrays: 16-byte aligned, a pitch that keeps rows 16-byte

@@ -1,9 +1,10 @@
 // One multigrid V(nu1, nu2) cycle (Sec. 3, Eqs. 19-24) enqueued on a stream.  Smoothing
-// per level: FP32 levels of aligned rows use the register-block kernel (two sweeps a pass, started
-// from zero without reading the iterate, the last pre-smoothing pass fused with the residual and
-// its full weighting); FP64 levels by size the row-marching kernel, the per-colour kernels or the
-// fused tile kernel (NS sweeps per launch, ping-pong iterates), then one kernel for the residual
-// fused with full-weighting restriction; the levels
+// per level: levels of aligned rows use the register-block kernel (FP32 all, FP64 small ones; two
+// sweeps a pass, started from zero without reading the iterate, the last pre-smoothing pass fused
+// with the residual and its full weighting); other FP64 levels by size the row-marching or the
+// per-colour kernels, rows without the alignment these or the fused tile kernel (NS sweeps per
+// launch, ping-pong iterates), then one kernel for the residual fused with full-weighting
+// restriction; the levels
 // at and below the tail threshold run in one single-CTA tail kernel that ends with the
 // coarsest dense solve.  The weighted-Jacobi smoother uses the per-sweep kernels on every
 // level, the zebra x-line smoother its two launches a sweep on every level but the coarsest.
@@ -68,6 +69,19 @@ int colour_nodes() {
   if (v < 0) {
     const char* e = getenv(sizeof(T) == 8 ? "MG_COLOUR_NODES_F64" : "MG_COLOUR_NODES_F32");
     v = e ? atoi(e) : 40000;
+  }
+  return v;
+}
+
+// FP64 levels of at most this many nodes use the register-block kernel.  Measured cycles (V(2,2), graph
+// replay) by the largest level it takes: 1025^2 with none 402 us, up to 129^2 348, 257^2 329, 513^2 365
+// (342 with one sweep a pass), 1025^2 544: on larger levels its redundant halo costs FP64 issue slots,
+// of which the per-colour kernels waste fewer; 129^2 cycle 127 -> 76 us.
+inline long long block_nodes_f64() {
+  static long long v = -1;
+  if (v < 0) {
+    const char* e = getenv("MG_BLOCK_NODES_F64");
+    v = e ? atoll(e) : 70000;
   }
   return v;
 }
@@ -235,7 +249,7 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
     // size-threshold rule, default variants.  FP32: register blocks were the fastest at every size
     // from 65^2 to 4097^2 (figures in k_block.cu), so size does not enter
     int kind, var = -1;
-    if (sizeof(T) == 4 && can(SK_BLOCK, -1))
+    if ((sizeof(T) == 4 || nodes <= block_nodes_f64()) && can(SK_BLOCK, -1))
       kind = SK_BLOCK;
     else if (sizeof(T) == 8 && nodes >= march_nodes() && can(SK_MARCH, -1))
       kind = SK_MARCH;
@@ -271,10 +285,9 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
       cur[l] = alt[l];
       alt[l] = tmp;
     };
-    if (kind == SK_BLOCK) {  // passes of block_sweeps<T>() sweeps, an odd one first
-      constexpr int NB = block_sweeps<T>();
+    if (kind == SK_BLOCK) {  // passes of two sweeps, an odd one first
       for (int left = sweeps; left > 0;) {
-        const int ns = left % NB ? 1 : NB;
+        const int ns = left % 2 ? 1 : 2;
         const bool first = left == sweeps, last = left == ns;
         err = launch_smooth_block<T>(V.A[l], first && zero ? nullptr : cur[l], alt[l], V.b[l], ns, rev,
                                      first ? eH : nullptr, last ? bH : nullptr, pc, skip, s);
