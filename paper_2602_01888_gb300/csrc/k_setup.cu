@@ -12,14 +12,15 @@ static const double kPi = 3.14159265358979323846;
 
 // eps = det(J) J^-1 (s I) J^-T for J = [[a, b], [c, d]] (Eqs. 10, 12-15).  cross = 0: a map
 // whose Eq. 13 vanishes identically (J^T J diagonal); eps_xy is then written as the exact
-// zero instead of the rounding residue of the general formula.
+// zero instead of the rounding residue of the general formula.  unit: s is 1.
 __device__ __forceinline__ void store_eps(double a, double b, double c, double d, double s,
                                           size_t k, double* D, double* exx, double* exy,
-                                          double* eyy, int* folded, int cross = 1) {
+                                          double* eyy, int* folded, int cross = 1, bool unit = false) {
   const double det = a * d - b * c;
-  if (!(det > 0.0)) atomicOr(folded, 1);
+  // det > 0, not NaN, from the bits: the comparison would run on the FP64 pipe
+  if ((unsigned long long)__double_as_longlong(det) - 1u >= 0x7ff0000000000000ull) atomicOr(folded, 1);
   D[k] = det;
-  const double sd = s / det;            // one division per node
+  const double sd = unit ? 1.0 / det : s / det;  // one division per node, cheaper as a reciprocal
   exx[k] = sd * (d * d + b * b);        // Eq. 12
   exy[k] = cross ? sd * (-d * c - b * a) : 0.0;  // Eq. 13 = Eq. 14
   eyy[k] = sd * (c * c + a * a);        // Eq. 15
@@ -97,7 +98,8 @@ __global__ void __launch_bounds__(256) k_eps_analytic(int kind, double p0, doubl
         break;
     }
     const size_t k = (size_t)j * pitch + i;
-    store_eps(a, b, c, d, eps ? eps[k] : 1.0, k, D, exx, exy, eyy, folded, cross);
+    if (eps) store_eps(a, b, c, d, eps[k], k, D, exx, exy, eyy, folded, cross);
+    else store_eps(a, b, c, d, 1.0, k, D, exx, exy, eyy, folded, cross, true);
   }
 }
 
@@ -148,6 +150,9 @@ __device__ __forceinline__ double ddy(const double* __restrict__ f, int i, int j
   return (f[(size_t)(j + 1) * pitch + i] - f[(size_t)(j - 1) * pitch + i]) * i2h;
 }
 
+// The inner nodes' four central differences stand in a branch of their own: inlined together, ddx and
+// ddy become predicated code, whose one-sided formulas take FP64 issue slots at every node (2049^2:
+// 294 -> 217 us; 27 FP64 operations a node, the pipe is the bound).
 __global__ void k_eps_grid(int nx, int ny, int nyr, int periodic, double i2hx, double i2hy,
                            const double* __restrict__ xp, const double* __restrict__ yp,
                            double jump_x, double jump_y, const double* __restrict__ eps,
@@ -157,11 +162,20 @@ __global__ void k_eps_grid(int nx, int ny, int nyr, int periodic, double i2hx, d
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= nx || j >= nyr) return;
   const size_t r = (size_t)j * pitch, k = r + i;
-  const double a = ddx(xp, r, i, nx, i2hx);                                  // Eq. 39
-  const double b = ddy(xp, i, j, ny, nyr, periodic, pitch, i2hy, jump_x);    // Eq. 40
-  const double c = ddx(yp, r, i, nx, i2hx);                                  // Eq. 41
-  const double d = ddy(yp, i, j, ny, nyr, periodic, pitch, i2hy, jump_y);    // Eq. 42
-  store_eps(a, b, c, d, eps ? eps[k] : 1.0, k, D, exx, exy, eyy, folded);
+  double a, b, c, d;
+  if (i > 0 && i < nx - 1 && j > 0 && j < nyr - 1) {  // the inner case of ddx and ddy
+    a = (xp[k + 1] - xp[k - 1]) * i2hx;          // Eq. 39
+    b = (xp[k + pitch] - xp[k - pitch]) * i2hy;  // Eq. 40
+    c = (yp[k + 1] - yp[k - 1]) * i2hx;          // Eq. 41
+    d = (yp[k + pitch] - yp[k - pitch]) * i2hy;  // Eq. 42
+  } else {
+    a = ddx(xp, r, i, nx, i2hx);
+    b = ddy(xp, i, j, ny, nyr, periodic, pitch, i2hy, jump_x);
+    c = ddx(yp, r, i, nx, i2hx);
+    d = ddy(yp, i, j, ny, nyr, periodic, pitch, i2hy, jump_y);
+  }
+  if (eps) store_eps(a, b, c, d, eps[k], k, D, exx, exy, eyy, folded);
+  else store_eps(a, b, c, d, 1.0, k, D, exx, exy, eyy, folded, 1, true);
 }
 
 // Couplings of the symmetric conservative 9-point operator A = -L_h.  five: eps_xy is zero
@@ -281,6 +295,86 @@ __global__ void __launch_bounds__(256) k_assemble_five(int nx, int ny, int nyr, 
       fdiag[kf] = dg;
       fdinv[kf] = 1.0f / dg;
     }
+  }
+}
+
+// One pass for a 9-point operator: the couplings of k_assemble_couplings, the diagonal, its
+// reciprocal (dinv when given) and, when fE is given, the FP32 copy with the reciprocal of the FP32
+// diagonal.  A warp covers 32 columns, of which it owns the inner 30, and marches down kAsmRows rows:
+// every tensor value is loaded once (shuffles and the row before give the neighbours').  The cross
+// couplings of a node cancel in the row sum, -q(i+1,j) - q(i,j+1) + q(i-1,j) + q(i,j+1) - q(i,j-1) -
+// q(i-1,j) + q(i,j-1) + q(i+1,j) = 0, so the diagonal is minus the sum of the E, W, N and S ones (three
+// roundings, as for a 5-point operator, instead of seven).  Bound by the FP64 pipe: 11 operations a
+// node and the five of dinv's reciprocal (15 and 5 with the cross terms in the sum): 157 us at
+// 2049^2, 197 us for the two separate kernels.
+constexpr int kAsmCols = 30;
+
+__global__ void __launch_bounds__(256) k_assemble_nine(int nx, int ny, int nyr, int periodic, int pitch, double mx,
+                                                       double my, double mxy, const double* __restrict__ exx,
+                                                       const double* __restrict__ exy,
+                                                       const double* __restrict__ eyy, double* cE, double* cN,
+                                                       double* cNE, double* cNW, double* diag, double* dinv, int pf,
+                                                       float* fE, float* fN, float* fNE, float* fNW, float* fdiag,
+                                                       float* fdinv) {
+  const int lane = threadIdx.x;
+  const int i = blockIdx.x * kAsmCols + lane - 1;
+  const int jb = (blockIdx.y * blockDim.y + threadIdx.y) * kAsmRows;
+  if (jb >= nyr) return;  // one strip per warp
+  const bool col = i >= 0 && i < nx, own = col && lane >= 1 && lane <= kAsmCols, has_e = i + 1 <= nx - 1;
+  auto get = [&](const double* __restrict__ f, int j) { return col ? f[(size_t)j * pitch + i] : 0.0; };
+  auto left = [](double v) { return __shfl_up_sync(0xffffffffu, v, 1); };
+  auto right = [](double v) { return __shfl_down_sync(0xffffffffu, v, 1); };
+  // couplings of row j to row j + 1 from the tensor values of the two rows
+  auto ups = [&](int j, double q, double y, double qu, double yu, double& n, double& ne, double& nw) {
+    const double ql = left(q), qr = right(q);
+    const bool up = col && (periodic || j + 1 <= ny - 1);
+    n = up ? __dmul_rn(__dadd_rn(y, yu), my) : 0.0;
+    ne = up && has_e ? __dmul_rn(__dadd_rn(qr, qu), -mxy) : 0.0;
+    nw = up && i >= 1 ? __dmul_rn(__dadd_rn(ql, qu), mxy) : 0.0;
+  };
+  double q = get(exy, jb), y = get(eyy, jb);
+  double ns = 0.0;  // coupling of the row below to this one
+  if (jb > 0 || periodic) {
+    const int jm = jb == 0 ? nyr - 1 : jb - 1;
+    ns = __dmul_rn(__dadd_rn(get(eyy, jm), y), my);
+  }
+  for (int r = 0; r < kAsmRows; ++r) {
+    const int j = jb + r;
+    if (j >= nyr) break;
+    const int ju = (j + 1 == nyr) ? 0 : j + 1;
+    const double x = get(exx, j), qu = get(exy, ju), yu = get(eyy, ju);
+    const double xr = right(x);
+    const double e = col && has_e ? __dmul_rn(__dadd_rn(x, xr), mx) : 0.0;
+    double n, ne, nw;
+    ups(j, q, y, qu, yu, n, ne, nw);
+    const double ew = left(e);
+    if (own) {
+      const size_t k = (size_t)j * pitch + i;
+      const bool unk = (i >= 1 && i <= nx - 2) && (periodic || (j >= 1 && j <= ny - 2));
+      double d = 1.0;
+      if (unk) {
+        d = -__dadd_rn(__dadd_rn(__dadd_rn(e, ew), n), ns);
+      }
+      cE[k] = e;
+      cN[k] = n;
+      cNE[k] = ne;
+      cNW[k] = nw;
+      diag[k] = d;
+      if (dinv) dinv[k] = unk ? 1.0 / d : 1.0;
+      if (fE) {
+        const size_t kf = (size_t)j * pf + i;
+        fE[kf] = (float)e;
+        fN[kf] = (float)n;
+        fNE[kf] = (float)ne;
+        fNW[kf] = (float)nw;
+        const float dg = (float)d;
+        fdiag[kf] = dg;
+        fdinv[kf] = 1.0f / dg;
+      }
+    }
+    q = qu;
+    y = yu;
+    ns = n;
   }
 }
 
@@ -407,6 +501,88 @@ __global__ void k_galerkin(Lvl<T> F, int nxc, int nyc, int nyrc, int pitchc, T* 
   cN[K] = row[1][2];
   cNE[K] = row[2][2];
   cNW[K] = row[0][2];
+}
+
+// The same product in FP64 collapsed first along x, then along y (P is the tensor product of the
+// one-dimensional interpolations): 62 FP64 operations a coarse node instead of 118.  Per fine row j
+// and coarse column I the first step gives h0, h1 (coupling of column I to itself and to I + 1
+// within the row) and u0, u1, um (to columns I, I + 1, I - 1 of the row above):
+//   h0 = d(2I) + (d(2I-1) + d(2I+1)) / 4 + E(2I-1) + E(2I)
+//   h1 = (E(2I) + E(2I+1)) / 2 + d(2I+1) / 4
+//   u0 = N(2I) + (N(2I-1) + N(2I+1)) / 4 + (NE(2I-1) + NE(2I) + NW(2I) + NW(2I+1)) / 2
+//   u1 = (NE(2I) + NE(2I+1)) / 2 + N(2I+1) / 4,   um = (NW(2I) + NW(2I-1)) / 2 + N(2I-1) / 4
+// and the second combines the rows 2J - 1, 2J, 2J + 1 the same way.  A warp holds 32 coarse columns,
+// of which it owns the inner 30 (the lanes beside supply E's and NW's missing halves), and marches
+// up a strip of coarse rows, so each fine row is collapsed once.  Pairs of columns are loaded as one
+// vector.  FIVE: zero NE / NW, whose terms vanish exactly.  Bound by the FP64 pipe (81% busy):
+// 2049^2 -> 1025^2 -> 513^2 220 us, 292 us with k_galerkin; rms error of the couplings against
+// 80-bit sums 2.1e-17 to 7.4e-17 of their largest, 2.2e-17 to 9.6e-17 before.
+constexpr int kGalCols = 30;
+
+struct GalRow {
+  double h0, h1, u0, u1, um;
+};
+
+template <bool FIVE>
+__global__ void __launch_bounds__(128, 5) k_galerkin_rows(Lvl<double> F, int nxc, int nyc, int nyrc, int pitchc, int rows,
+                                                       double* __restrict__ cE, double* __restrict__ cN,
+                                                       double* __restrict__ cNE, double* __restrict__ cNW,
+                                                       double* __restrict__ diag, double* __restrict__ dinv) {
+  const int lane = threadIdx.x & 31;
+  const int I = blockIdx.x * kGalCols + lane - 1;
+  const int Jb = (blockIdx.y * (blockDim.x / 32) + (threadIdx.x >> 5)) * rows, Je = min(Jb + rows, nyrc);
+  if (Jb >= nyrc) return;  // one strip per warp
+  const bool col = I >= 0 && I < nxc, own = col && lane >= 1 && lane <= kGalCols;
+  auto left = [](double v) { return __shfl_up_sync(0xffffffffu, v, 1); };
+  auto right = [](double v) { return __shfl_down_sync(0xffffffffu, v, 1); };
+  auto row = [&](int j) -> GalRow {  // j wrapped or clamped into the grid by the caller
+    const size_t k = (size_t)j * F.pitch + 2 * I;
+    const double2 z = make_double2(0.0, 0.0);
+    auto get = [&](const double* a) { return col ? __ldg(reinterpret_cast<const double2*>(a + k)) : z; };
+    const double2 d = get(F.diag), e = get(F.cE), n = get(F.cN);
+    const double dl = left(d.y), el = left(e.y), nl = left(n.y);
+    GalRow g;
+    g.h0 = fma(0.25, dl + d.y, d.x) + (el + e.x);
+    g.h1 = fma(0.5, e.x + e.y, 0.25 * d.y);
+    g.u0 = fma(0.25, nl + n.y, n.x);
+    if (FIVE) {
+      g.u1 = 0.25 * n.y;
+      g.um = 0.25 * nl;
+    } else {
+      const double2 ne = get(F.cNE), nw = get(F.cNW);
+      const double nel = left(ne.y), nwl = left(nw.y);
+      g.u0 = fma(0.5, (nel + ne.x) + (nw.x + nw.y), g.u0);
+      g.u1 = fma(0.5, ne.x + ne.y, 0.25 * n.y);
+      g.um = fma(0.5, nw.x + nwl, 0.25 * nl);
+    }
+    return g;
+  };
+  auto fine = [&](int j) { return F.periodic ? (j < 0 ? j + F.nyr : (j >= F.nyr ? j - F.nyr : j)) : min(max(j, 0), F.nyr - 1); };
+  GalRow p = row(fine(2 * Jb - 1));
+  for (int J = Jb; J < Je; ++J) {
+    const GalRow c = row(fine(2 * J)), n = row(fine(2 * J + 1));
+    const double s_um = right(p.um + c.um);  // um of column I + 1
+    const double h1l = left(n.h1);           // h1 of column I - 1
+    if (own) {
+      const size_t K = (size_t)J * pitchc + I;
+      const bool unk = I >= 1 && I <= nxc - 2 && (F.periodic || (J >= 1 && J <= nyc - 2));
+      double vE = 0.0, vN = 0.0, vNE = 0.0, vNW = 0.0, vd = 1.0;
+      if (unk) {
+        vd = 0.25 * (fma(0.25, p.h0 + n.h0, c.h0) + (p.u0 + c.u0));
+        vE = 0.25 * fma(0.5, (p.u1 + c.u1) + s_um, fma(0.25, p.h1 + n.h1, c.h1));
+        vN = 0.25 * fma(0.5, c.u0 + n.u0, 0.25 * n.h0);
+        vNE = 0.25 * fma(0.5, c.u1 + n.u1, 0.25 * n.h1);
+        vNW = 0.25 * fma(0.5, c.um + n.um, 0.25 * h1l);
+      }
+      diag[K] = vd;
+      dinv[K] = unk ? 1.0 / vd : 1.0;
+      cE[K] = vE;
+      cN[K] = vN;
+      cNE[K] = vNE;
+      cNW[K] = vNW;
+    }
+    p = n;
+  }
 }
 
 __global__ void k_op_to_f32(int nx, int nyr, int ps, int pd, const double* __restrict__ a0,
@@ -539,6 +715,9 @@ cudaError_t launch_eps_grid(int nx, int ny, int periodic, double hx, double hy, 
 template <typename T>
 cudaError_t launch_assemble(const Op<T>& A, double hx, double hy, const T* exx, const T* exy, const T* eyy,
                             cudaStream_t s, bool dinv) {
+  if constexpr (sizeof(T) == 8) {
+    if (!A.five_point) return launch_assemble_nine(A, nullptr, hx, hy, exx, exy, eyy, s, dinv);
+  }
   const int nyr = rows_stored(A.ny, A.periodic);
   dim3 b(32, 8);
   k_assemble_couplings<T><<<grid2(A.nx, nyr, b), b, 0, s>>>(
@@ -553,6 +732,17 @@ template cudaError_t launch_assemble<double>(const OpF64&, double, double, const
                                              const double*, cudaStream_t, bool);
 template cudaError_t launch_assemble<float>(const OpF32&, double, double, const float*, const float*,
                                             const float*, cudaStream_t, bool);
+
+cudaError_t launch_assemble_nine(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
+                                 const double* exy, const double* eyy, cudaStream_t s, bool dinv) {
+  const int nyr = rows_stored(A.ny, A.periodic);
+  dim3 b(32, 8), g((A.nx + kAsmCols - 1) / kAsmCols, (nyr + 8 * kAsmRows - 1) / (8 * kAsmRows));
+  k_assemble_nine<<<g, b, 0, s>>>(
+      A.nx, A.ny, nyr, A.periodic, A.pitch, -0.5 * (1.0 / (hx * hx)), -0.5 * (1.0 / (hy * hy)), 1.0 / (4.0 * hx * hy), exx,
+      exy, eyy, A.cE, A.cN, A.cNE, A.cNW, A.diag, dinv ? A.dinv : nullptr, B ? B->pitch : 0, B ? B->cE : nullptr,
+      B ? B->cN : nullptr, B ? B->cNE : nullptr, B ? B->cNW : nullptr, B ? B->diag : nullptr, B ? B->dinv : nullptr);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_assemble_five(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
                                  const double* eyy, cudaStream_t s, bool dinv) {
@@ -595,6 +785,23 @@ template cudaError_t launch_coarsen_eps<float, float>(const OpF32&, const OpF32&
 template <typename T>
 cudaError_t launch_galerkin(const Op<T>& F, const Op<T>& C, cudaStream_t s) {
   const int nyrc = rows_stored(C.ny, C.periodic);
+  if constexpr (sizeof(T) == 8) {
+    const uintptr_t all = (uintptr_t)F.cE | (uintptr_t)F.cN | (uintptr_t)F.cNE | (uintptr_t)F.cNW | (uintptr_t)F.diag;
+    if (F.pitch % 2 == 0 && all % 16 == 0) {  // rows readable in pairs of columns
+      // strips of eight coarse rows (one more fine row collapsed per strip: 6%), shorter on small
+      // levels, whose few warps would leave SMs idle
+      const int gx = (C.nx + kGalCols - 1) / kGalCols;
+      const int rows = (long long)gx * nyrc > 8LL * 152 * 16 ? 8 : 2;
+      const dim3 g(gx, (nyrc + 4 * rows - 1) / (4 * rows));
+      if (F.five_point)
+        k_galerkin_rows<true><<<g, 128, 0, s>>>(lvl_of(F), C.nx, C.ny, nyrc, C.pitch, rows, C.cE, C.cN, C.cNE, C.cNW,
+                                                C.diag, C.dinv);
+      else
+        k_galerkin_rows<false><<<g, 128, 0, s>>>(lvl_of(F), C.nx, C.ny, nyrc, C.pitch, rows, C.cE, C.cN, C.cNE, C.cNW,
+                                                 C.diag, C.dinv);
+      return cudaGetLastError();
+    }
+  }
   dim3 b(32, 4);
   if (F.five_point)
     k_galerkin<T, true><<<grid2(C.nx, nyrc, b), b, 0, s>>>(lvl_of(F), C.nx, C.ny, nyrc, C.pitch, C.cE,

@@ -94,6 +94,9 @@ cudaError_t launch_assemble(const Op<T>& A, double hx, double hy, const T* exx, 
 // values.  dinv: write A's FP64 reciprocal diagonal.
 cudaError_t launch_assemble_five(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
                                  const double* eyy, cudaStream_t s, bool dinv);
+// launch_assemble for a 9-point FP64 operator, with the same FP32 copy when B is given.
+cudaError_t launch_assemble_nine(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
+                                 const double* exy, const double* eyy, cudaStream_t s, bool dinv);
 cudaError_t launch_rhs(const OpF64& A, const double* rho, int rho_pitch, const double* D, double* b,
                        cudaStream_t s);
 template <typename T>

@@ -439,12 +439,14 @@ mg_status problem_enqueue_build(mg_problem* P, const mg_map_desc* map, const dou
     eyy = P->p;
   }
   // a mixed hierarchy never runs an FP64 smoother: its level-0 reciprocal diagonal is the FP32
-  // one, taken from the FP32 diagonal, so the FP64 division per node is skipped.  Without a
-  // cross term (and without a caller's change of the finest operator, which the FP32 copy
-  // must follow) couplings, diagonal and the FP32 copy come from one pass.
-  const bool five_pass = F.A.five_point && !(hook && *hook);
-  const bool f32_done = five_pass && P->mixed;
-  if (five_pass) CU(launch_assemble_five(F.A, P->mixed ? &F.A32 : nullptr, hx, hy, exx, eyy, s, !P->mixed));
+  // one, taken from the FP32 diagonal, so the FP64 division per node is skipped.  Couplings,
+  // diagonal and the FP32 copy come from one pass (without the copy if a caller changes the finest
+  // operator, which the copy must follow).
+  const bool hooked = hook && *hook;
+  const bool f32_done = P->mixed && !hooked;
+  const OpF32* const copy = f32_done ? &F.A32 : nullptr;
+  if (F.A.five_point && !hooked) CU(launch_assemble_five(F.A, copy, hx, hy, exx, eyy, s, !P->mixed));
+  else if (!F.A.five_point) CU(launch_assemble_nine(F.A, copy, hx, hy, exx, exy, eyy, s, !P->mixed));
   else CU(launch_assemble(F.A, hx, hy, exx, exy, eyy, s, !P->mixed));
   if (hook && *hook) {  // a caller's change of the finest operator before coarsening
     mg_status hs = (*hook)(P, s);
@@ -501,12 +503,11 @@ mg_status problem_enqueue_build(mg_problem* P, const mg_map_desc* map, const dou
     if (P->nlev > 1) CU(launch_op_to_f64(P->lev[P->nlev - 1].A32, P->lev[P->nlev - 1].A, s));
   }
   CU(launch_coarse_factor(P->lev[P->nlev - 1].A, P->inv, P->flags + 1, s));
-  P->setup_kernels =
-      P->coarse_op == MG_COARSE_REDISCRETIZE
-          ? 1 + 2 + 3 * (P->nlev - 1) + (P->mixed ? 1 + (P->nlev > 1 ? 1 : 0) : 0) + 1 + (P->mirror ? 1 : 0)
-          : 1 + 2 + (P->mixed ? 1 + (P->nlev - 1) + (P->nlev > 1 ? 1 : 0) : P->nlev - 1) + 1 +
-                (P->mirror ? 1 : 0);
-  if (five_pass) P->setup_kernels -= f32_done ? 2 : 1;  // one kernel for two (three with the FP32 copy)
+  // tensor (and its reflection), finest operator, FP32 copy, coarse levels, coarsest inverse
+  const int coarse_kernels =  // per level: Galerkin product, or coarsened tensor and its assembly
+      P->coarse_op == MG_COARSE_REDISCRETIZE ? (P->mixed || F.A.five_point ? 3 : 2) : 1;
+  P->setup_kernels = 1 + (P->mirror ? 1 : 0) + (F.A.five_point && hooked ? 2 : 1) + (P->mixed && !f32_done ? 1 : 0) +
+                     coarse_kernels * (P->nlev - 1) + (P->mixed && P->nlev > 1 ? 1 : 0) + 1;
   if (P->line) {  // the line smoother's row factors follow the new operators
     mg_status ls = line_enqueue_factor(P, s, &P->setup_kernels);
     if (ls) return ls;
