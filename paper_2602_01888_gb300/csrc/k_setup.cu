@@ -10,96 +10,123 @@ namespace mg {
 
 static const double kPi = 3.14159265358979323846;
 
-// eps = det(J) J^-1 (s I) J^-T for J = [[a, b], [c, d]] (Eqs. 10, 12-15).  cross = 0: a map
-// whose Eq. 13 vanishes identically (J^T J diagonal); eps_xy is then written as the exact
-// zero instead of the rounding residue of the general formula.  unit: s is 1.
-__device__ __forceinline__ void store_eps(double a, double b, double c, double d, double s,
-                                          size_t k, double* D, double* exx, double* exy,
-                                          double* eyy, int* folded, int cross = 1, bool unit = false) {
-  const double det = a * d - b * c;
-  // det > 0, not NaN, from the bits: the comparison would run on the FP64 pipe
-  if ((unsigned long long)__double_as_longlong(det) - 1u >= 0x7ff0000000000000ull) atomicOr(folded, 1);
-  D[k] = det;
-  const double sd = unit ? 1.0 / det : s / det;  // one division per node, cheaper as a reciprocal
-  exx[k] = sd * (d * d + b * b);        // Eq. 12
-  exy[k] = cross ? sd * (-d * c - b * a) : 0.0;  // Eq. 13 = Eq. 14
-  eyy[k] = sd * (c * c + a * a);        // Eq. 15
+// Whether det J is zero, negative or NaN, from the bits: a comparison would run on the FP64 pipe.
+__device__ __forceinline__ bool folds(double det) {
+  return (unsigned long long)__double_as_longlong(det) - 1u >= 0x7ff0000000000000ull;
 }
 
-// One CTA per 32 x 32 tile of nodes (32 x 8 threads, four rows each).  Every analytic map's
-// Jacobian is built from transcendental factors of x alone and of y alone, so they are
-// evaluated once per column and once per row of the tile, in shared memory, rather than once
-// per node: FP64 transcendentals, not memory traffic, bound this kernel otherwise.  The
-// factors are the same calls on the same arguments as a per-node evaluation, so the results
-// do not change.
+// eps = det(J) J^-1 (s I) J^-T for J = [[a, b], [c, d]] (Eqs. 10, 12-15); unit: s is 1.
+__device__ __forceinline__ void store_eps(double a, double b, double c, double d, double s,
+                                          size_t k, double* D, double* exx, double* exy,
+                                          double* eyy, int* folded, bool unit) {
+  const double det = a * d - b * c;
+  if (folds(det)) atomicOr(folded, 1);
+  D[k] = det;
+  const double sd = unit ? 1.0 / det : s / det;  // one division per node, cheaper as a reciprocal
+  exx[k] = sd * (d * d + b * b);     // Eq. 12
+  exy[k] = sd * (-d * c - b * a);    // Eq. 13 = Eq. 14
+  eyy[k] = sd * (c * c + a * a);     // Eq. 15
+}
+
+// One CTA per 32 x 32 tile of nodes (32 x 8 threads, four rows each).  The sine warp's Jacobian is
+// built from transcendental factors of x alone and of y alone, so they are evaluated once per column
+// and once per row of the tile, in shared memory, rather than once per node: FP64 transcendentals,
+// not memory traffic, bound this kernel otherwise.
 constexpr int kEpsTile = 32;
 
-__global__ void __launch_bounds__(256) k_eps_analytic(int kind, double p0, double p1, double p2,
-                                                      double p3, int nx, int nyr, double x0, double y0,
-                                                      double hx, double hy,
-                                                      const double* __restrict__ eps, int pitch,
-                                                      double* D, double* exx, double* exy, double* eyy,
-                                                      int* folded, int cross) {
+__global__ void __launch_bounds__(256) k_eps_sine_warp(double p0, int nx, int nyr, double x0, double y0,
+                                                       double hx, double hy,
+                                                       const double* __restrict__ eps, int pitch,
+                                                       double* D, double* exx, double* exy, double* eyy,
+                                                       int* folded) {
   __shared__ double colv[4][kEpsTile], rowv[2][kEpsTile];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i0 = blockIdx.x * kEpsTile, j0 = blockIdx.y * kEpsTile;
   if (ty == 0) {  // factors of x
     const double x = x0 + (i0 + tx) * hx;
-    if (kind == 1) {
-      sincos(kPi * x, &colv[0][tx], &colv[1][tx]);
-      sincos(2.0 * kPi * x, &colv[2][tx], &colv[3][tx]);
-    } else if (kind == 3) {
-      colv[0][tx] = cosh(p1 * x);
-    }
+    sincos(kPi * x, &colv[0][tx], &colv[1][tx]);
+    sincos(2.0 * kPi * x, &colv[2][tx], &colv[3][tx]);
   } else if (ty == 1) {  // factors of y
     const double y = y0 + (j0 + tx) * hy;
-    if (kind == 1) sincos(kPi * y, &rowv[0][tx], &rowv[1][tx]);
-    else if (kind == 2) sincos(y, &rowv[0][tx], &rowv[1][tx]);
-    else if (kind == 3) rowv[0][tx] = cosh(p1 * y);
+    sincos(kPi * y, &rowv[0][tx], &rowv[1][tx]);
   }
   __syncthreads();
   const int i = i0 + tx;
   if (i >= nx) return;
-  const double x = x0 + i * hx;
+  const double sx = colv[0][tx], cx = colv[1][tx], s2x = colv[2][tx], c2x = colv[3][tx];
 #pragma unroll
   for (int r = 0; r < kEpsTile / 8; ++r) {
     const int ly = ty + 8 * r, j = j0 + ly;
     if (j >= nyr) break;
-    double a = 1.0, b = 0.0, c = 0.0, d = 1.0;  // Jxx Jxy Jyx Jyy
-    switch (kind) {
-      case 1: {  // sine warp
-        const double sx = colv[0][tx], cx = colv[1][tx], s2x = colv[2][tx], c2x = colv[3][tx];
-        const double sy = rowv[0][ly], cy = rowv[1][ly];
-        a = 1.0 + p0 * kPi * cx * sy;
-        b = p0 * kPi * sx * cy;
-        c = p0 * 2.0 * kPi * c2x * sy;
-        d = 1.0 + p0 * kPi * s2x * cy;
-        break;
-      }
-      case 2: {  // polar, Eq. 29
-        const double sy = rowv[0][ly], cy = rowv[1][ly];
-        a = cy;
-        b = -x * sy;
-        c = sy;
-        d = x * cy;
-        break;
-      }
-      case 3:  // sinh stretching, Eq. 52
-        a = p0 * p1 * colv[0][tx];
-        d = p0 * p1 * rowv[0][ly];
-        break;
-      case 4:  // affine
-        a = p0;
-        b = p1;
-        c = p2;
-        d = p3;
-        break;
-      default:
-        break;
-    }
+    const double sy = rowv[0][ly], cy = rowv[1][ly];
+    const double a = 1.0 + p0 * kPi * cx * sy;  // Jxx
+    const double b = p0 * kPi * sx * cy;        // Jxy
+    const double c = p0 * 2.0 * kPi * c2x * sy;  // Jyx
+    const double d = 1.0 + p0 * kPi * s2x * cy;  // Jyy
     const size_t k = (size_t)j * pitch + i;
-    if (eps) store_eps(a, b, c, d, eps[k], k, D, exx, exy, eyy, folded, cross);
-    else store_eps(a, b, c, d, 1.0, k, D, exx, exy, eyy, folded, cross, true);
+    if (eps) store_eps(a, b, c, d, eps[k], k, D, exx, exy, eyy, folded, false);
+    else store_eps(a, b, c, d, 1.0, k, D, exx, exy, eyy, folded, true);
+  }
+}
+
+// The other analytic maps, whose Eqs. 10, 12-15 are a factor of x times a factor of y:
+//   polar (Eq. 29)   D = x                     eps_xx = s x                  eps_yy = s / x
+//   sinh (Eq. 52)    D = a(x) d(y)             eps_xx = s (1 / a) d          eps_yy = s a (1 / d)
+//   affine, identity D, eps_xx / s, eps_xy / s and eps_yy / s constant (cD, cxx, cxy, cyy)
+// with a = p0 p1 cosh(p1 x), d = p0 p1 cosh(p1 y).  The factors are evaluated once per column and row
+// of a tile of 32 x 32 nodes; a node costs two products and no division (ROWS, factors of y: five),
+// so the 32 or 40 bytes it moves bound the kernel (polar 8193 x 8192 without s: 291 us, 7.4 TB/s).  Through
+// the general formula the FP64 pipe did, with a division a node (2604 us).  cross = 0: Eq. 13 vanishes identically, eps_xy is zero.
+template <bool ROWS>
+__global__ void __launch_bounds__(256) k_eps_separable(int kind, double p0, double p1, double cD, double cxx,
+                                                       double cxy, double cyy, int nx, int nyr, double x0, double y0,
+                                                       double hx, double hy, const double* __restrict__ eps, int pitch,
+                                                       double* __restrict__ D, double* __restrict__ exx,
+                                                       double* __restrict__ exy, double* __restrict__ eyy, int* folded,
+                                                       int cross) {
+  __shared__ double colv[2][kEpsTile], rowv[2][kEpsTile];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int i0 = blockIdx.x * kEpsTile, j0 = blockIdx.y * kEpsTile;
+  if (kind == 2 || kind == 3) {
+    if (ty == 0) {
+      const double x = x0 + (i0 + tx) * hx;
+      const double f = kind == 2 ? x : p0 * p1 * cosh(p1 * x);
+      colv[0][tx] = f;
+      colv[1][tx] = 1.0 / f;
+    } else if (ROWS && ty == 1) {
+      const double f = p0 * p1 * cosh(p1 * (y0 + (j0 + tx) * hy));
+      rowv[0][tx] = f;
+      rowv[1][tx] = 1.0 / f;
+    }
+    __syncthreads();
+  }
+  const int i = i0 + tx;
+  if (i >= nx) return;
+  double fD = cD, fx = cxx, fy = cyy;
+  if (kind == 2) {
+    fD = fx = colv[0][tx];
+    fy = colv[1][tx];
+  } else if (kind == 3) {
+    fD = fy = colv[0][tx];
+    fx = colv[1][tx];
+  }
+#pragma unroll
+  for (int r = 0; r < kEpsTile / 8; ++r) {
+    const int ly = ty + 8 * r, j = j0 + ly;
+    if (j >= nyr) break;
+    const size_t k = (size_t)j * pitch + i;
+    double det = fD, gx = fx, gy = fy;
+    if (ROWS) {
+      det *= rowv[0][ly];
+      gx *= rowv[0][ly];
+      gy *= rowv[1][ly];
+    }
+    if (folds(det)) atomicOr(folded, 1);
+    D[k] = det;
+    const double s = eps ? eps[k] : 1.0;
+    exx[k] = s * gx;                   // Eq. 12
+    exy[k] = cross ? s * cxy : 0.0;    // Eq. 13 = Eq. 14
+    eyy[k] = s * gy;                   // Eq. 15
   }
 }
 
@@ -174,8 +201,8 @@ __global__ void k_eps_grid(int nx, int ny, int nyr, int periodic, double i2hx, d
     c = ddx(yp, r, i, nx, i2hx);
     d = ddy(yp, i, j, ny, nyr, periodic, pitch, i2hy, jump_y);
   }
-  if (eps) store_eps(a, b, c, d, eps[k], k, D, exx, exy, eyy, folded);
-  else store_eps(a, b, c, d, 1.0, k, D, exx, exy, eyy, folded, 1, true);
+  if (eps) store_eps(a, b, c, d, eps[k], k, D, exx, exy, eyy, folded, false);
+  else store_eps(a, b, c, d, 1.0, k, D, exx, exy, eyy, folded, true);
 }
 
 // Couplings of the symmetric conservative 9-point operator A = -L_h.  five: eps_xy is zero
@@ -688,8 +715,16 @@ cudaError_t launch_eps_analytic(int kind, const double* prm, int nx, int ny, int
                                 int* folded, cudaStream_t s) {
   const int nyr = rows_stored(ny, periodic);
   dim3 b(32, 8), g((nx + kEpsTile - 1) / kEpsTile, (nyr + kEpsTile - 1) / kEpsTile);
-  k_eps_analytic<<<g, b, 0, s>>>(kind, prm[0], prm[1], prm[2], prm[3], nx, nyr, x0, y0, hx, hy, eps, pitch,
-                                 D, exx, exy, eyy, folded, map_kind_five_point(kind, prm) ? 0 : 1);
+  if (kind == 1) {
+    k_eps_sine_warp<<<g, b, 0, s>>>(prm[0], nx, nyr, x0, y0, hx, hy, eps, pitch, D, exx, exy, eyy, folded);
+    return cudaGetLastError();
+  }
+  const double ja = kind == 4 ? prm[0] : 1.0, jb = kind == 4 ? prm[1] : 0.0, jc = kind == 4 ? prm[2] : 0.0,
+               jd = kind == 4 ? prm[3] : 1.0, det = ja * jd - jb * jc;
+  const auto f = kind == 3 ? k_eps_separable<true> : k_eps_separable<false>;
+  f<<<g, b, 0, s>>>(kind, prm[0], prm[1], det, (jd * jd + jb * jb) / det, (-jd * jc - jb * ja) / det,
+                    (jc * jc + ja * ja) / det, nx, nyr, x0, y0, hx, hy, eps, pitch, D, exx, exy, eyy, folded,
+                    map_kind_five_point(kind, prm) ? 0 : 1);
   return cudaGetLastError();
 }
 

@@ -1,7 +1,8 @@
 """Set-up kernels that do in one pass what several did: the 9-point assembly (a warp owns 30
 columns and marches strips of 8 rows), its couplings and its diagonal (four terms, the cross ones
 cancel) bit for bit and against the sum over all eight couplings, and the row-collapsed FP64 Galerkin product (30 coarse columns a warp) against the oracle and, on rows of
-an odd pitch, against the direct product, at sizes around those edges."""
+an odd pitch, against the direct product, and the analytic maps whose tensor is a factor of x times a
+factor of y against the general formula (tiles of 32 x 32), at sizes around those edges."""
 import ctypes as C
 
 import numpy as np
@@ -80,3 +81,40 @@ def test_row_collapsed_galerkin(libmg, oracle, cuda, shape, five):
     # both sum the same products of magnitude up to 8 in different orders: 1e-14 absolute
     for a, b in zip(*got):
         assert np.abs(a - b).max() <= 1e-14
+
+
+MAPS = {"identity": (0, (0.0,) * 4), "polar": (2, (0.0,) * 4), "sinh": (3, (0.7, 1.3, 0.0, 0.0)),
+        "scaled": (4, (1.5, 0.0, 0.0, 0.75)), "sheared": (4, (1.1, 0.2, -0.1, 0.9))}
+
+
+@pytest.mark.parametrize("name", list(MAPS))
+@pytest.mark.parametrize("nx,ny,per,physical", [(5, 5, 0, 1), (31, 33, 0, 0), (32, 65, 1, 1), (67, 31, 0, 1)])
+def test_separable_maps(libmg, cuda, name, nx, ny, per, physical):
+    torch = cuda
+    kind, prm = MAPS[name]
+    nyr, pitch, x0, y0, hx, hy = (ny - 1 if per else ny), nx + 3, 1.0, 0.25, 1.0 / (nx - 1), 2.0 / (ny - 1)
+    s = np.random.default_rng(nx).uniform(0.5, 8.0, (nyr, nx)) if physical else np.ones((nyr, nx))
+    x, y = (x0 + np.arange(nx) * hx)[None, :] + np.zeros((nyr, 1)), (y0 + np.arange(nyr) * hy)[:, None] + np.zeros((1, nx))
+    p, one, zero = prm, np.ones_like(x), np.zeros_like(x)
+    a, b, c, d = {0: (one, zero, zero, one), 2: (np.cos(y), -x * np.sin(y), np.sin(y), x * np.cos(y)),
+                  3: (p[0] * p[1] * np.cosh(p[1] * x), zero, zero, p[0] * p[1] * np.cosh(p[1] * y)),
+                  4: (p[0] * one, p[1] * one, p[2] * one, p[3] * one)}[kind]
+    det = a * d - b * c
+    ref = [det, s / det * (d * d + b * b), s / det * (-d * c - b * a), s / det * (c * c + a * a)]
+    put = lambda v: torch.nn.functional.pad(torch.from_numpy(v), (0, pitch - nx)).contiguous().cuda()
+    eps = put(s) if physical else None
+    out = [torch.full((nyr, pitch), 7.0, dtype=torch.float64, device="cuda") for _ in range(4)]
+    folded = torch.zeros(1, dtype=torch.int32, device="cuda")
+    libmg.mgk("mgk_eps_analytic", kind, (C.c_double * 4)(*prm), nx, ny, per, x0, y0, hx, hy,
+              eps.data_ptr() if physical else None, pitch, *[v.data_ptr() for v in out], folded.data_ptr(),
+              torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert int(folded.item()) == 0
+    got = [v.cpu().numpy() for v in out]
+    emag = max(np.abs(ref[1]).max(), np.abs(ref[3]).max())
+    # at most 16 roundings a side (two of them cosh's two units), none in a cancelling sum but exy's
+    for v, r, m in zip(got, ref, (det.max(), emag, emag, emag)):
+        assert np.abs(v[:, :nx] - r).max() <= 32 * 2.0 ** -53 * m
+        assert (v[:, nx:] == 7.0).all()
+    if name != "sheared":
+        assert (got[2][:, :nx] == 0.0).all()
