@@ -69,16 +69,59 @@ __global__ void __launch_bounds__(256) k_eps_sine_warp(double p0, int nx, int ny
   }
 }
 
+// Polar map (Eq. 29), the general formula with what depends on one coordinate taken out of the node:
+// the row's sum of squares, and 1 / x for the division.  det J = x (cos^2 + sin^2) is x but for
+// rounding, so one Newton step from 1 / x gives 1 / det to one rounding.  The closed form (D = x,
+// eps_xx = s x, eps_yy = s / x) would be cheaper still, but its rounding is the same at every node of
+// a circle and adds up in the row sums of the operator: at 8193^2 it moves the solution by 3e-10.
+// Ten FP64 operations a node bound it: 8193 x 8192 1.43 ms, 2.60 ms with the division and the sums at
+// every node.
+__global__ void __launch_bounds__(256) k_eps_polar(int nx, int nyr, double x0, double y0, double hx, double hy,
+                                                   const double* __restrict__ eps, int pitch,
+                                                   double* __restrict__ D, double* __restrict__ exx,
+                                                   double* __restrict__ exy, double* __restrict__ eyy, int* folded) {
+  __shared__ double colv[kEpsTile], rowv[3][kEpsTile];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int i0 = blockIdx.x * kEpsTile, j0 = blockIdx.y * kEpsTile;
+  if (ty == 0) colv[tx] = 1.0 / (x0 + (i0 + tx) * hx);
+  if (ty == 1) {
+    double c, a;
+    sincos(y0 + (j0 + tx) * hy, &c, &a);
+    rowv[0][tx] = c;
+    rowv[1][tx] = a;
+    rowv[2][tx] = c * c + a * a;
+  }
+  __syncthreads();
+  const int i = i0 + tx;
+  if (i >= nx) return;
+  const double x = x0 + i * hx, rx = colv[tx];
+#pragma unroll
+  for (int r = 0; r < kEpsTile / 8; ++r) {
+    const int ly = ty + 8 * r, j = j0 + ly;
+    if (j >= nyr) break;
+    const double c = rowv[0][ly], a = rowv[1][ly];  // Jyx, Jxx
+    const double b = -x * c, d = x * a;             // Jxy, Jyy
+    const double det = a * d - b * c;
+    if (folds(det)) atomicOr(folded, 1);
+    const size_t k = (size_t)j * pitch + i;
+    D[k] = det;
+    double sd = fma(rx, fma(-det, rx, 1.0), rx);
+    if (eps) sd *= eps[k];
+    exx[k] = sd * (d * d + b * b);  // Eq. 12
+    exy[k] = 0.0;                   // Eq. 13 vanishes identically
+    eyy[k] = sd * rowv[2][ly];      // Eq. 15
+  }
+}
+
 // The other analytic maps, whose Eqs. 10, 12-15 are a factor of x times a factor of y:
-//   polar (Eq. 29)   D = x                     eps_xx = s x                  eps_yy = s / x
 //   sinh (Eq. 52)    D = a(x) d(y)             eps_xx = s (1 / a) d          eps_yy = s a (1 / d)
 //   affine, identity D, eps_xx / s, eps_xy / s and eps_yy / s constant (cD, cxx, cxy, cyy)
 // with a = p0 p1 cosh(p1 x), d = p0 p1 cosh(p1 y).  The factors are evaluated once per column and row
-// of a tile of 32 x 32 nodes; a node costs two products and no division (ROWS, factors of y: five),
-// so the 32 or 40 bytes it moves bound the kernel (polar 8193 x 8192 without s: 291 us, 7.4 TB/s).  Through
-// the general formula the FP64 pipe did, with a division a node (2604 us).  cross = 0: Eq. 13 vanishes identically, eps_xy is zero.
-template <bool ROWS>
-__global__ void __launch_bounds__(256) k_eps_separable(int kind, double p0, double p1, double cD, double cxx,
+// of a tile of 32 x 32 nodes; a node costs two products and no division (SINH: five), so the 32 or 40
+// bytes it moves bound the kernel.  Through the general formula the FP64 pipe did, with a division a
+// node.  cross = 0: Eq. 13 vanishes identically, eps_xy is zero.
+template <bool SINH>
+__global__ void __launch_bounds__(256) k_eps_separable(double p0, double p1, double cD, double cxx,
                                                        double cxy, double cyy, int nx, int nyr, double x0, double y0,
                                                        double hx, double hy, const double* __restrict__ eps, int pitch,
                                                        double* __restrict__ D, double* __restrict__ exx,
@@ -87,36 +130,26 @@ __global__ void __launch_bounds__(256) k_eps_separable(int kind, double p0, doub
   __shared__ double colv[2][kEpsTile], rowv[2][kEpsTile];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i0 = blockIdx.x * kEpsTile, j0 = blockIdx.y * kEpsTile;
-  if (kind == 2 || kind == 3) {
-    if (ty == 0) {
-      const double x = x0 + (i0 + tx) * hx;
-      const double f = kind == 2 ? x : p0 * p1 * cosh(p1 * x);
-      colv[0][tx] = f;
-      colv[1][tx] = 1.0 / f;
-    } else if (ROWS && ty == 1) {
-      const double f = p0 * p1 * cosh(p1 * (y0 + (j0 + tx) * hy));
-      rowv[0][tx] = f;
-      rowv[1][tx] = 1.0 / f;
+  double fD = cD, fx = cxx, fy = cyy;
+  if (SINH) {
+    if (ty < 2) {
+      const double f = p0 * p1 * cosh(p1 * (ty == 0 ? x0 + (i0 + tx) * hx : y0 + (j0 + tx) * hy));
+      (ty == 0 ? colv : rowv)[0][tx] = f;
+      (ty == 0 ? colv : rowv)[1][tx] = 1.0 / f;
     }
     __syncthreads();
-  }
-  const int i = i0 + tx;
-  if (i >= nx) return;
-  double fD = cD, fx = cxx, fy = cyy;
-  if (kind == 2) {
-    fD = fx = colv[0][tx];
-    fy = colv[1][tx];
-  } else if (kind == 3) {
     fD = fy = colv[0][tx];
     fx = colv[1][tx];
   }
+  const int i = i0 + tx;
+  if (i >= nx) return;
 #pragma unroll
   for (int r = 0; r < kEpsTile / 8; ++r) {
     const int ly = ty + 8 * r, j = j0 + ly;
     if (j >= nyr) break;
     const size_t k = (size_t)j * pitch + i;
     double det = fD, gx = fx, gy = fy;
-    if (ROWS) {
+    if (SINH) {
       det *= rowv[0][ly];
       gx *= rowv[0][ly];
       gy *= rowv[1][ly];
@@ -719,10 +752,14 @@ cudaError_t launch_eps_analytic(int kind, const double* prm, int nx, int ny, int
     k_eps_sine_warp<<<g, b, 0, s>>>(prm[0], nx, nyr, x0, y0, hx, hy, eps, pitch, D, exx, exy, eyy, folded);
     return cudaGetLastError();
   }
+  if (kind == 2) {
+    k_eps_polar<<<g, b, 0, s>>>(nx, nyr, x0, y0, hx, hy, eps, pitch, D, exx, exy, eyy, folded);
+    return cudaGetLastError();
+  }
   const double ja = kind == 4 ? prm[0] : 1.0, jb = kind == 4 ? prm[1] : 0.0, jc = kind == 4 ? prm[2] : 0.0,
                jd = kind == 4 ? prm[3] : 1.0, det = ja * jd - jb * jc;
   const auto f = kind == 3 ? k_eps_separable<true> : k_eps_separable<false>;
-  f<<<g, b, 0, s>>>(kind, prm[0], prm[1], det, (jd * jd + jb * jb) / det, (-jd * jc - jb * ja) / det,
+  f<<<g, b, 0, s>>>(prm[0], prm[1], det, (jd * jd + jb * jb) / det, (-jd * jc - jb * ja) / det,
                     (jc * jc + ja * ja) / det, nx, nyr, x0, y0, hx, hy, eps, pitch, D, exx, exy, eyy, folded,
                     map_kind_five_point(kind, prm) ? 0 : 1);
   return cudaGetLastError();
