@@ -347,11 +347,11 @@ __global__ void __launch_bounds__(256) k_assemble_five(int nx, int ny, int nyr, 
     if (dinv) dinv[k] = unk ? 1.0 / d : 1.0;
     if (fE) {
       const size_t kf = (size_t)j * pf + i;
-      fE[kf] = (float)e;
-      fN[kf] = (float)n;
+      fE[kf] = narrow(e);
+      fN[kf] = narrow(n);
       fNE[kf] = 0.0f;
       fNW[kf] = 0.0f;
-      const float dg = (float)d;
+      const float dg = narrow(d);
       fdiag[kf] = dg;
       fdinv[kf] = 1.0f / dg;
     }
@@ -423,11 +423,11 @@ __global__ void __launch_bounds__(256) k_assemble_nine(int nx, int ny, int nyr, 
       if (dinv) dinv[k] = unk ? 1.0 / d : 1.0;
       if (fE) {
         const size_t kf = (size_t)j * pf + i;
-        fE[kf] = (float)e;
-        fN[kf] = (float)n;
-        fNE[kf] = (float)ne;
-        fNW[kf] = (float)nw;
-        const float dg = (float)d;
+        fE[kf] = narrow(e);
+        fN[kf] = narrow(n);
+        fNE[kf] = narrow(ne);
+        fNW[kf] = narrow(nw);
+        const float dg = narrow(d);
         fdiag[kf] = dg;
         fdinv[kf] = 1.0f / dg;
       }
@@ -654,13 +654,13 @@ __global__ void k_op_to_f32(int nx, int nyr, int ps, int pd, const double* __res
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= nx || j >= nyr) return;
   const size_t s = (size_t)j * ps + i, d = (size_t)j * pd + i;
-  b0[d] = (float)a0[s];
-  b1[d] = (float)a1[s];
-  b2[d] = five ? 0.0f : (float)a2[s];  // a 5-point operator's NE / NW are zero: not read
-  b3[d] = five ? 0.0f : (float)a3[s];
-  const float dg = (float)a4[s];
+  b0[d] = narrow(a0[s]);
+  b1[d] = narrow(a1[s]);
+  b2[d] = five ? 0.0f : narrow(a2[s]);  // a 5-point operator's NE / NW are zero: not read
+  b3[d] = five ? 0.0f : narrow(a3[s]);
+  const float dg = narrow(a4[s]);
   b4[d] = dg;
-  b5[d] = dinv_f32 ? 1.0f / dg : (float)a5[s];  // dinv_f32: reciprocal of the FP32 diagonal
+  b5[d] = dinv_f32 ? 1.0f / dg : narrow(a5[s]);  // dinv_f32: reciprocal of the FP32 diagonal
 }
 
 // Dense matrix of the coarsest level's unknowns, inverted by Gauss-Jordan elimination

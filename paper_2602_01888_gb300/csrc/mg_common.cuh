@@ -92,31 +92,82 @@ struct SolveState {
 
 static_assert(sizeof(SolveState) % 8 == 0, "SolveState is copied as 8-byte words");
 
+// ---- FP32 <-> FP64 on the integer pipe ---------------------------------------------
+// GB300 converts between FP32 and FP64 on its FP64 pipe, which takes some 60 cycles an instruction
+// and warp; the same values from the bits of the two IEEE 754 formats take about ten instructions of
+// two cycles.  Every value but a NaN converts as the cast does (to nearest, ties to even); a NaN
+// stays one.
+struct Bits64 {
+  unsigned hi, lo;
+};
+
+__host__ __device__ __forceinline__ Bits64 widen_bits(unsigned mag, unsigned sign, bool tiny) {
+  // mag: exponent and fraction bits, of the value times 2^64 if tiny (below the normal range)
+  const unsigned rebias = tiny ? 0x34000000u : (mag >= 0x7f800000u ? 0x70000000u : 0x38000000u);
+  return {(mag ? (mag >> 3) + rebias : 0u) | sign, mag << 29};
+}
+
+__device__ __forceinline__ double widen(float v) {
+  const bool tiny = (__float_as_uint(v) & 0x7f800000u) == 0;
+  const unsigned u = __float_as_uint(tiny ? v * 0x1p64f : v);
+  const Bits64 b = widen_bits(u & 0x7fffffffu, u & 0x80000000u, tiny);
+  return __hiloint2double((int)b.hi, (int)b.lo);
+}
+
+// Magnitude bits of the nearest float outside its normal range: overflow, infinity, NaN, or a
+// multiple of 2^-149 below 2^-126.
+__host__ __device__ __forceinline__ unsigned narrow_far(unsigned mag, unsigned lo) {
+  if (mag >= 0x47f00000u) return mag > 0x7ff00000u || (mag == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u;
+  const unsigned sh = 926u - (mag >> 20);  // from units of 2^(e - 1075) to 2^-149; at least 30
+  if (sh >= 54u) return 0u;
+  const unsigned long long m = ((unsigned long long)((mag & 0xfffffu) | 0x100000u) << 32) | lo;
+  const unsigned long long q = m >> sh, rem = m & ((1ull << sh) - 1);
+  return (unsigned)(q + (rem + (q & 1) > (1ull << (sh - 1)) ? 1 : 0));
+}
+
+__host__ __device__ __forceinline__ unsigned narrow_bits(unsigned hi, unsigned lo) {
+  const unsigned mag = hi & 0x7fffffffu;
+  unsigned f = ((mag - 0x38000000u) << 3) | (lo >> 29);
+  f += (lo & 0x1fffffffu) + (f & 1u) > 0x10000000u ? 1u : 0u;
+  if (mag - 0x38100000u >= 0x0fe00000u) f = narrow_far(mag, lo);
+  return f | (hi & 0x80000000u);
+}
+
+__device__ __forceinline__ float narrow(double v) {
+  return __uint_as_float(narrow_bits((unsigned)__double2hiint(v), (unsigned)__double2loint(v)));
+}
+
 // ---- deterministic block reduction -------------------------------------------------
-// Sums each of the K values of v over the block in a fixed order (warp shuffle tree, then warps in
-// order, one lane per value); valid in thread 0.
+// Sums each of the K values of v over the block in a fixed order (warp q adds value q's NT / 32
+// columns of shared memory, then its lanes in a shuffle tree); valid in thread 0.  A tree in every
+// warp first would take 40 FP64 instructions a value where this takes 12: they are the scarce ones.
 template <int NT, int K>
-__device__ __forceinline__ void block_sums(double (&v)[K], double* sh /* >= K NT/32 */) {
+constexpr int kSumsShared = K * NT + K;
+
+template <int NT, int K>
+__device__ __forceinline__ void block_sums(double (&v)[K], double* sh /* kSumsShared<NT, K> */) {
   constexpr int NW = NT / 32;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int q = 0; q < K; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+  static_assert(K <= NW && (NW & (NW - 1)) == 0, "one warp per value, a power of two of columns");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
 #pragma unroll
-    for (int q = 0; q < K; ++q) sh[q * NW + warp] = v[q];
+  for (int q = 0; q < K; ++q) sh[q * NT + threadIdx.x] = v[q];
   __syncthreads();
-  if (warp == 0) {
-    double t = 0.0;
-    if (lane < K) {
+  if (warp < K) {
+    double t[NW];
 #pragma unroll
-      for (int w = 0; w < NW; ++w) t += sh[lane * NW + w];
-    }
+    for (int w = 0; w < NW; ++w) t[w] = sh[warp * NT + w * 32 + lane];
 #pragma unroll
-    for (int q = 0; q < K; ++q) v[q] = __shfl_sync(0xffffffffu, t, q);
+    for (int n = NW / 2; n > 0; n >>= 1)
+#pragma unroll
+      for (int w = 0; w < n; ++w) t[w] += t[w + n];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t[0] += __shfl_down_sync(0xffffffffu, t[0], o);
+    if (lane == 0) sh[K * NT + warp] = t[0];
   }
   __syncthreads();
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int q = 0; q < K; ++q) v[q] = sh[K * NT + q];
 }
 
 // After thread 0 of each block has written the block's partial sums, the block that arrives last
@@ -143,17 +194,19 @@ __device__ __forceinline__ void reduce_partials(const double* part, int n, doubl
   constexpr int B = 8;
 #pragma unroll
   for (int q = 0; q < K; ++q) v[q] = 0.0;
-  for (int k0 = threadIdx.x; k0 < n; k0 += B * NT) {
+  for (int base = 0; base < n; base += B * NT) {
+    const int k0 = base + threadIdx.x;
     double w[K][B];
 #pragma unroll
     for (int q = 0; q < K; ++q)
 #pragma unroll
       for (int u = 0; u < B; ++u) w[q][u] = k0 + u * NT < n ? __ldcg(part + (size_t)q * n + k0 + u * NT) : 0.0;
 #pragma unroll
-    for (int q = 0; q < K; ++q)
+    for (int u = 0; u < B; ++u) {
+      if (base + u * NT >= n) break;  // uniform: no FP64 issue slots for rows past the end
 #pragma unroll
-      for (int u = 0; u < B; ++u)
-        if (k0 + u * NT < n) v[q] += w[q][u];
+      for (int q = 0; q < K; ++q) v[q] += w[q][u];
+    }
   }
   block_sums<NT, K>(v, sh);
 }

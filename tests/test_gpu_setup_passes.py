@@ -1,8 +1,9 @@
 """Set-up kernels that do in one pass what several did: the 9-point assembly (a warp owns 30
 columns and marches strips of 8 rows), its couplings and its diagonal (four terms, the cross ones
-cancel) bit for bit and against the sum over all eight couplings, and the row-collapsed FP64 Galerkin product (30 coarse columns a warp) against the oracle and, on rows of
-an odd pitch, against the direct product, and the analytic maps whose tensor is a factor of x times a
-factor of y against the general formula (tiles of 32 x 32), at sizes around those edges."""
+cancel) bit for bit and against the sum over all eight couplings; the row-collapsed FP64 Galerkin
+product (30 coarse columns a warp) against the direct product, which rows of an odd pitch take;
+and the analytic maps with factors of one coordinate (tiles of 32 x 32) against the general
+formula.  Sizes around those edges."""
 import ctypes as C
 
 import numpy as np
