@@ -26,7 +26,7 @@
 // 203 -> 164 us (row marching).  Marching a strip with everything in one warp's registers, without
 // any barrier, was slower (177 us at 4097^2, 18 us at 1025^2: two warps a scheduler cannot hide the
 // chain of a step).  FP64 (32 x 32 regions, two CTAs an SM) is bound by a phase's chain of ten FP64
-// operations: two sweeps with the restriction or the correction take about 12 us at 65^2 and 129^2,
+// operations: two sweeps with the restriction or the correction take about 11 us at 65^2 and 129^2,
 // where the fused tile kernel took 18 us without either.
 //
 // Operations per node and their order are those of the per-colour kernels and of
@@ -295,10 +295,15 @@ __global__ void __launch_bounds__(TX * TY, BlockGeom<T, NS, TX, TY, RR>::CTAS)
     if constexpr (RR) {
       const T* const d = dg + buf * ARR;
       const P2 g0 = *reinterpret_cast<const P2*>(d + o0), g1 = *reinterpret_cast<const P2*>(d + o1);
-      const T ra = ma ? b0.x - fma(g0.x, xa, sum_a()) : T(0);
-      const T rb = mb ? b0.y - fma(g0.y, xb, sum_b()) : T(0);
-      const T rc = mc ? b1.x - fma(g1.x, xc, sum_c()) : T(0);
-      const T rd = md ? b1.y - fma(g1.y, xd, sum_d()) : T(0);
+      // at the owned nodes and one block row and column before them
+      const bool used = 2 * ty >= G::HB - 2 && 2 * ty < RY - G::HT;
+      T ra = T(0), rb = T(0), rc = T(0), rd = T(0);
+      if (used) {
+        if (ma) ra = b0.x - fma(g0.x, xa, sum_a());
+        if (mb) rb = b0.y - fma(g0.y, xb, sum_b());
+        if (mc) rc = b1.x - fma(g1.x, xc, sum_c());
+        if (md) rd = b1.y - fma(g1.y, xd, sum_d());
+      }
       T* const Rb = rp + ty * TX + tx;
       T* const Rc = Rb + PL;
       T* const Rd = Rc + PL;

@@ -141,24 +141,40 @@ __global__ void __launch_bounds__(kREven) k_resid_restrict_even(Lvl<T> L, const 
   if (xH) xH[K] = T(0);
 }
 
-// x += P eH (bilinear: injection at coincident nodes, 1/2 on edges, 1/4 at centres).
-template <typename T>
+// x += P eH (bilinear: injection at coincident nodes, 1/2 on edges, 1/4 at centres).  A thread corrects
+// the 2 x 2 fine nodes up and right of a coarse node: eight operations for the four, without the
+// divergence of one thread a node (in FP64 five issue slots a node, on the pipe that bounds it):
+// FP64 1025^2 14.9 -> 9.4 us.  VEC: pairs of columns in one access.
+template <typename T, bool VEC>
 __global__ void __launch_bounds__(256) k_prolong_add(Lvl<T> L, T* __restrict__ x,
-                                                     const T* __restrict__ eH, int nyrc,
+                                                     const T* __restrict__ eH, int nxc, int nyrc,
                                                      int pitchc, const int* __restrict__ skip) {
   if (skip && *skip) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (!is_unknown(L, i, j)) return;
-  const int I = i >> 1, J = j >> 1;
-  const int Jp = (J + 1 == nyrc) ? 0 : J + 1;
-  const size_t a = (size_t)J * pitchc + I, c = (size_t)Jp * pitchc + I;
-  T v;
-  if (!(i & 1) && !(j & 1)) v = eH[a];
-  else if ((i & 1) && !(j & 1)) v = T(0.5) * (eH[a] + eH[a + 1]);
-  else if (!(i & 1)) v = T(0.5) * (eH[a] + eH[c]);
-  else v = T(0.25) * ((eH[a] + eH[a + 1]) + (eH[c] + eH[c + 1]));
-  x[(size_t)j * L.pitch + i] += v;
+  const int I = blockIdx.x * blockDim.x + threadIdx.x;
+  const int J = blockIdx.y * blockDim.y + threadIdx.y;
+  if (I >= nxc || J >= nyrc) return;
+  const int i = 2 * I, j = 2 * J;
+  const size_t a = (size_t)J * pitchc + I, c = (size_t)(J + 1 == nyrc ? 0 : J + 1) * pitchc + I;
+  const T ea = eH[a], ec = eH[c];
+  const bool e = I + 1 < nxc;
+  const T eb = e ? eH[a + 1] : T(0), ed = e ? eH[c + 1] : T(0);
+  const T lo = ea + eb, le = ea + ec, all = lo + (ec + ed);
+  T* const p = x + (size_t)j * L.pitch + i;
+  auto row = [&](T* q, int jj, T d0, T h, T w) {  // q[0] += d0, q[1] += w h at the unknowns of row jj
+    const bool u0 = is_unknown(L, i, jj), u1 = is_unknown(L, i + 1, jj);
+    if (VEC && u0 && u1) {
+      using P = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+      P v = *reinterpret_cast<P*>(q);
+      v.x += d0;
+      v.y = fma(w, h, v.y);
+      *reinterpret_cast<P*>(q) = v;
+    } else {
+      if (u0) q[0] += d0;
+      if (u1) q[1] = fma(w, h, q[1]);
+    }
+  };
+  row(p, j, ea, lo, T(0.5));
+  row(p + L.pitch, j + 1, T(0.5) * le, all, T(0.25));
 }
 
 // x = inv * b at the coarsest unknowns (lexicographic, i fastest), one CTA.
@@ -273,10 +289,13 @@ template <typename T>
 cudaError_t launch_prolong_add(const Op<T>& A, T* phi, const T* eH, int pitch_c, const int* skip,
                                cudaStream_t s) {
   const Lvl<T> L = lvl_of(A);
-  const int nyc = (A.ny - 1) / 2 + 1;
+  const int nxc = (A.nx - 1) / 2 + 1, nyrc = rows_stored((A.ny - 1) / 2 + 1, A.periodic);
   dim3 bl(32, 8);
-  k_prolong_add<T><<<g2(L.nx, L.nyr, bl), bl, 0, s>>>(L, phi, eH, rows_stored(nyc, A.periodic),
-                                                      pitch_c, skip);
+  const dim3 g = g2(nxc, nyrc, bl);
+  if (A.pitch % 2 == 0 && (uintptr_t)phi % (2 * sizeof(T)) == 0)
+    k_prolong_add<T, true><<<g, bl, 0, s>>>(L, phi, eH, nxc, nyrc, pitch_c, skip);
+  else
+    k_prolong_add<T, false><<<g, bl, 0, s>>>(L, phi, eH, nxc, nyrc, pitch_c, skip);
   return cudaGetLastError();
 }
 

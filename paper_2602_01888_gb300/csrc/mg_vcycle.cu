@@ -73,15 +73,17 @@ int colour_nodes() {
   return v;
 }
 
-// FP64 levels of at most this many nodes use the register-block kernel.  Measured cycles (V(2,2), graph
-// replay) by the largest level it takes: 1025^2 with none 402 us, up to 129^2 348, 257^2 329, 513^2 365
-// (342 with one sweep a pass), 1025^2 544: on larger levels its redundant halo costs FP64 issue slots,
-// of which the per-colour kernels waste fewer; 129^2 cycle 127 -> 76 us.
+// FP64 levels of at most this many nodes use the register-block kernel: those whose 22 x 16 tiles the
+// GPU holds at once (304).  Measured cycles (V(2,2), graph replay) by the largest level it takes: 1025^2
+// with none 402 us, up to 129^2 348, 257^2 329, 513^2 365, 1025^2 544 (since then 317 up to 257^2);
+// 1537 x 1025 up to 193 x 129 552 us, 385 x 257 518.  On larger levels the redundant halo costs FP64
+// issue slots, of which the per-colour kernels waste fewer: taller tiles (22 x 48) did not change that
+// (1025^2 with 513^2 in them 342 us, against 322 at the time).
 inline long long block_nodes_f64() {
   static long long v = -1;
   if (v < 0) {
     const char* e = getenv("MG_BLOCK_NODES_F64");
-    v = e ? atoll(e) : 70000;
+    v = e ? atoll(e) : 107008;
   }
   return v;
 }
