@@ -562,11 +562,17 @@ __global__ void __launch_bounds__(kNT) k_copy_out(Lvl<double> L, const double* _
 }
 
 // ------------------------------------------------------------------ launchers
+// One column a thread and, beyond a block an SM, four rows or more a block: a block's sums cost as much
+// FP64 work as a row of it, and solves that share the GPU share that pipe (batch of 64, sides 65 to 513:
+// 20.7 ms with one row a block, 18.6 with two, 17.6 with four, 17.9 with eight); on one small grid alone
+// (129^2) one row a block on every SM is the faster split (0.874 ms against 0.882 with two).
 dim3 red_grid(int nx, int nyr) {
   const int gx = (nx + kNT - 1) / kNT;
   int gy = kRedBlocks / gx;
   if (gy < 1) gy = 1;
-  if (gy > nyr) gy = nyr;
+  const int fewest = (152 + gx - 1) / gx, spread = (nyr + 3) / 4;
+  const int most = spread > fewest ? spread : (fewest < nyr ? fewest : nyr);
+  if (gy > most) gy = most;
   return dim3(gx, gy);
 }
 
