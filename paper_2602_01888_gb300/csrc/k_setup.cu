@@ -295,81 +295,24 @@ __global__ void k_assemble_diag(int nx, int ny, int nyr, int periodic, int pitch
   if (dinv) dinv[k] = T(1) / (-s);
 }
 
-// One pass for an operator without cross term (5-point, eps_xy = 0): the E and N couplings
-// of k_assemble_couplings, the diagonal (and its reciprocal when dinv is given) of
-// k_assemble_diag and, when fE is given, the FP32 copy of k_op_to_f32 with the reciprocal of
-// the FP32 diagonal (pitch pf).  A warp covers 32 columns of a row and each thread marches
-// down kAsmRows rows: the coupling to the W neighbour is the left lane's E coupling (shuffle),
-// the one to the S neighbour the thread's N coupling of the row before; the first lane and the
-// first row of a strip compute theirs again.  A coupling is rounded like the separate
-// kernel's: -(1/2)(a + b) / h^2 is the sum times the exact constant -(1/2) / h^2 (halving is
-// exact), one rounding per operation (__dadd_rn, __dmul_rn: no contracted multiply-add), so
-// the values are bitwise those of the separate kernels.  NE / NW get zeros, as from
-// k_assemble_couplings, for the kernels that have no 5-point form.  GB300 issues FP64 at a
-// low rate: ten FP64 operations per node here, as many as the three separate kernels take.
+// One pass over the finest level: the couplings of k_assemble_couplings, the diagonal, its reciprocal
+// (dinv when given) and, when fE is given, the FP32 copy of k_op_to_f32 with the reciprocal of the FP32
+// diagonal (pitch pf).  A warp covers 32 columns, of which it owns the inner 30, and marches down
+// kAsmRows rows: every tensor value is loaded once (shuffles and the row before give the
+// neighbours').  A coupling is rounded like the separate kernel's: -(1/2)(a + b) / h^2 is the sum times
+// the exact constant -(1/2) / h^2 (halving is exact), one rounding per operation (__dadd_rn,
+// __dmul_rn: no contracted multiply-add), so the couplings are bitwise those of the separate kernels.
+// The cross couplings of a node cancel in the row sum, -q(i+1,j) - q(i,j+1) + q(i-1,j) + q(i,j+1) -
+// q(i,j-1) - q(i-1,j) + q(i,j-1) + q(i+1,j) = 0, so the diagonal is minus the sum of the E, W, N and S
+// ones (three roundings instead of seven).  FIVE: eps_xy is zero everywhere; NE / NW get zeros, for
+// the kernels that have no 5-point form.  Bound by the FP64 pipe: 11 operations a node (FIVE: 7) and
+// the five of dinv's reciprocal.  9-point 2049^2 157 us, 197 us with the two separate kernels; 5-point
+// 8193^2 with the FP32 copy 1.33 -> 1.22 ms (every first lane computed its W coupling, predicated).
 constexpr int kAsmRows = 8;
-
-__global__ void __launch_bounds__(256) k_assemble_five(int nx, int ny, int nyr, int periodic, int pitch, double mx,
-                                                       double my, const double* __restrict__ exx,
-                                                       const double* __restrict__ eyy, double* cE, double* cN,
-                                                       double* cNE, double* cNW, double* diag, double* dinv, int pf,
-                                                       float* fE, float* fN, float* fNE, float* fNW, float* fdiag,
-                                                       float* fdinv) {
-  const int i = blockIdx.x * 32 + threadIdx.x;
-  const int jb = (blockIdx.y * blockDim.y + threadIdx.y) * kAsmRows;
-  const bool col = i < nx;
-  const bool has_e = i + 1 <= nx - 1;
-  double n_prev = 0.0;
-  for (int r = 0; r < kAsmRows; ++r) {
-    const int j = jb + r;
-    if (j >= nyr) break;  // the same for the whole warp (one row per warp)
-    const size_t k = (size_t)j * pitch + i;
-    const int ju = (j + 1 == nyr) ? 0 : j + 1;
-    const double e = (col && has_e) ? __dmul_rn(__dadd_rn(exx[k], exx[k + 1]), mx) : 0.0;
-    const double n = (col && (periodic || j + 1 <= ny - 1))
-                         ? __dmul_rn(__dadd_rn(eyy[k], eyy[(size_t)ju * pitch + i]), my) : 0.0;
-    double ew = __shfl_up_sync(0xffffffffu, e, 1);
-    double ns = n_prev;
-    n_prev = n;
-    if (!col) continue;
-    const bool unk = (i >= 1 && i <= nx - 2) && (periodic || (j >= 1 && j <= ny - 2));
-    double d = 1.0;
-    if (unk) {
-      if (threadIdx.x == 0) ew = __dmul_rn(__dadd_rn(exx[k - 1], exx[k]), mx);
-      if (r == 0) ns = __dmul_rn(__dadd_rn(eyy[(size_t)((j == 0) ? nyr - 1 : j - 1) * pitch + i], eyy[k]), my);
-      d = -__dadd_rn(__dadd_rn(__dadd_rn(e, ew), n), ns);
-    }
-    cE[k] = e;
-    cN[k] = n;
-    cNE[k] = 0.0;
-    cNW[k] = 0.0;
-    diag[k] = d;
-    if (dinv) dinv[k] = unk ? 1.0 / d : 1.0;
-    if (fE) {
-      const size_t kf = (size_t)j * pf + i;
-      fE[kf] = narrow(e);
-      fN[kf] = narrow(n);
-      fNE[kf] = 0.0f;
-      fNW[kf] = 0.0f;
-      const float dg = narrow(d);
-      fdiag[kf] = dg;
-      fdinv[kf] = 1.0f / dg;
-    }
-  }
-}
-
-// One pass for a 9-point operator: the couplings of k_assemble_couplings, the diagonal, its
-// reciprocal (dinv when given) and, when fE is given, the FP32 copy with the reciprocal of the FP32
-// diagonal.  A warp covers 32 columns, of which it owns the inner 30, and marches down kAsmRows rows:
-// every tensor value is loaded once (shuffles and the row before give the neighbours').  The cross
-// couplings of a node cancel in the row sum, -q(i+1,j) - q(i,j+1) + q(i-1,j) + q(i,j+1) - q(i,j-1) -
-// q(i-1,j) + q(i,j-1) + q(i+1,j) = 0, so the diagonal is minus the sum of the E, W, N and S ones (three
-// roundings, as for a 5-point operator, instead of seven).  Bound by the FP64 pipe: 11 operations a
-// node and the five of dinv's reciprocal (15 and 5 with the cross terms in the sum): 157 us at
-// 2049^2, 197 us for the two separate kernels.
 constexpr int kAsmCols = 30;
 
-__global__ void __launch_bounds__(256) k_assemble_nine(int nx, int ny, int nyr, int periodic, int pitch, double mx,
+template <bool FIVE>
+__global__ void __launch_bounds__(256) k_assemble_pass(int nx, int ny, int nyr, int periodic, int pitch, double mx,
                                                        double my, double mxy, const double* __restrict__ exx,
                                                        const double* __restrict__ exy,
                                                        const double* __restrict__ eyy, double* cE, double* cN,
@@ -386,13 +329,15 @@ __global__ void __launch_bounds__(256) k_assemble_nine(int nx, int ny, int nyr, 
   auto right = [](double v) { return __shfl_down_sync(0xffffffffu, v, 1); };
   // couplings of row j to row j + 1 from the tensor values of the two rows
   auto ups = [&](int j, double q, double y, double qu, double yu, double& n, double& ne, double& nw) {
-    const double ql = left(q), qr = right(q);
     const bool up = col && (periodic || j + 1 <= ny - 1);
     n = up ? __dmul_rn(__dadd_rn(y, yu), my) : 0.0;
+    ne = nw = 0.0;
+    if (FIVE) return;
+    const double ql = left(q), qr = right(q);
     ne = up && has_e ? __dmul_rn(__dadd_rn(qr, qu), -mxy) : 0.0;
     nw = up && i >= 1 ? __dmul_rn(__dadd_rn(ql, qu), mxy) : 0.0;
   };
-  double q = get(exy, jb), y = get(eyy, jb);
+  double q = FIVE ? 0.0 : get(exy, jb), y = get(eyy, jb);
   double ns = 0.0;  // coupling of the row below to this one
   if (jb > 0 || periodic) {
     const int jm = jb == 0 ? nyr - 1 : jb - 1;
@@ -402,7 +347,7 @@ __global__ void __launch_bounds__(256) k_assemble_nine(int nx, int ny, int nyr, 
     const int j = jb + r;
     if (j >= nyr) break;
     const int ju = (j + 1 == nyr) ? 0 : j + 1;
-    const double x = get(exx, j), qu = get(exy, ju), yu = get(eyy, ju);
+    const double x = get(exx, j), qu = FIVE ? 0.0 : get(exy, ju), yu = get(eyy, ju);
     const double xr = right(x);
     const double e = col && has_e ? __dmul_rn(__dadd_rn(x, xr), mx) : 0.0;
     double n, ne, nw;
@@ -805,27 +750,27 @@ template cudaError_t launch_assemble<double>(const OpF64&, double, double, const
 template cudaError_t launch_assemble<float>(const OpF32&, double, double, const float*, const float*,
                                             const float*, cudaStream_t, bool);
 
-cudaError_t launch_assemble_nine(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
+// -(1/2) / h^2 exactly (halving is exact), as k_assemble_couplings rounds its couplings
+template <bool FIVE>
+static cudaError_t assemble_pass(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
                                  const double* exy, const double* eyy, cudaStream_t s, bool dinv) {
   const int nyr = rows_stored(A.ny, A.periodic);
   dim3 b(32, 8), g((A.nx + kAsmCols - 1) / kAsmCols, (nyr + 8 * kAsmRows - 1) / (8 * kAsmRows));
-  k_assemble_nine<<<g, b, 0, s>>>(
+  k_assemble_pass<FIVE><<<g, b, 0, s>>>(
       A.nx, A.ny, nyr, A.periodic, A.pitch, -0.5 * (1.0 / (hx * hx)), -0.5 * (1.0 / (hy * hy)), 1.0 / (4.0 * hx * hy), exx,
       exy, eyy, A.cE, A.cN, A.cNE, A.cNW, A.diag, dinv ? A.dinv : nullptr, B ? B->pitch : 0, B ? B->cE : nullptr,
       B ? B->cN : nullptr, B ? B->cNE : nullptr, B ? B->cNW : nullptr, B ? B->diag : nullptr, B ? B->dinv : nullptr);
   return cudaGetLastError();
 }
 
+cudaError_t launch_assemble_nine(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
+                                 const double* exy, const double* eyy, cudaStream_t s, bool dinv) {
+  return assemble_pass<false>(A, B, hx, hy, exx, exy, eyy, s, dinv);
+}
+
 cudaError_t launch_assemble_five(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
                                  const double* eyy, cudaStream_t s, bool dinv) {
-  const int nyr = rows_stored(A.ny, A.periodic);
-  dim3 b(32, 8), g((A.nx + 31) / 32, (nyr + 8 * kAsmRows - 1) / (8 * kAsmRows));
-  // -(1/2) / h^2 exactly (halving is exact), as k_assemble_couplings rounds its couplings
-  k_assemble_five<<<g, b, 0, s>>>(
-      A.nx, A.ny, nyr, A.periodic, A.pitch, -0.5 * (1.0 / (hx * hx)), -0.5 * (1.0 / (hy * hy)), exx, eyy, A.cE, A.cN, A.cNE,
-      A.cNW, A.diag, dinv ? A.dinv : nullptr, B ? B->pitch : 0, B ? B->cE : nullptr, B ? B->cN : nullptr,
-      B ? B->cNE : nullptr, B ? B->cNW : nullptr, B ? B->diag : nullptr, B ? B->dinv : nullptr);
-  return cudaGetLastError();
+  return assemble_pass<true>(A, B, hx, hy, exx, nullptr, eyy, s, dinv);
 }
 
 cudaError_t launch_rhs(const OpF64& A, const double* rho, int rho_pitch, const double* D, double* b,
