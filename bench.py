@@ -48,7 +48,7 @@ def _hbm_peak():
 
 
 HBM_PEAK_GBS, HBM_PEAK_SOURCE = _hbm_peak()
-MARCH_NODES = 2000000  # FP32 levels of at least this many nodes are smoothed by the marching kernel
+MARCH_NODES = 2000000  # untuned FP64 levels of at least this many nodes are smoothed by the marching kernel
 
 
 def _traffic_table():
@@ -447,8 +447,8 @@ def _fp64_roof(mg, torch, kern, tflops, launch_s, g, **extra):
 def measure_smoother(mg, torch, inst, prec, reps=20, smoother="gs4", family=None):
     """Dominant kernel of the level-0 smoothing timed alone with CUDA events on this
     workload's finest level, operator built by the library's own kernels: one four-colour
-    Gauss-Seidel sweep (4 launches of k_gs_colour), or on FP32 levels of at least
-    MARCH_NODES nodes one launch of the row-marching kernel (two sweeps).  FP64: flop-bound
+    Gauss-Seidel sweep (4 launches of k_gs_colour), or on FP32 levels one launch of the
+    register-block kernel (two sweeps).  FP64: flop-bound
     (18 flop per updated unknown); FP32: bytes-bound (algorithmic 32 B per node and pass:
     iterate read and written, b, four couplings, 1/diag)."""
     import ctypes as C
@@ -491,7 +491,7 @@ def measure_smoother(mg, torch, inst, prec, reps=20, smoother="gs4", family=None
         return _measure_line(mg, torch, g, st, x, b, f32, s, reps, five)
     fam, shape = parse_choice(family)
     if fam is None:  # untuned: the size rule of the cycle
-        fam = "marching" if g.nx * g.nyr >= MARCH_NODES else "colour"
+        fam = "marching" if f32 or g.nx * g.nyr >= MARCH_NODES else "colour"
     if fam in ("pipelined", "fused", "marching"):
         return _measure_variant(mg, torch, g, st, x, z(dt), b, f32, s, reps, fam, shape)
 
@@ -567,7 +567,8 @@ def _measure_variant(mg, torch, g, st, x, x2, b, f32, s, reps, family, shape):
     per_launch_s = e0.elapsed_time(e1) * 1e-3 / reps
     T = "float" if f32 else "double"
     if family == "marching":
-        kern = f"k_smooth_march<{T}> w{tile[0]}/{ns}"  # owned strip columns / sweeps per pass
+        # owned columns of a tile or strip / sweeps per pass; the register blocks are the narrow ones
+        kern = f"k_smooth_{'block' if tile[0] == (52 if f32 else 22) else 'march'}<{T}> w{tile[0]}/{ns}"
     else:
         kern = f"k_smooth_{'pipe' if family == 'pipelined' else 'fused'}<{T},{tile[0]},{tile[1]},{ns}>"
     note = f"the autotuner's choice for this level size ({family}), {ns} sweep(s) per launch"
@@ -637,8 +638,9 @@ def _measure_line(mg, torch, g, st, x, b, f32, s, reps, five=False):
     e1.record()
     torch.cuda.synchronize()
     per_launch_s = e0.elapsed_time(e1) * 1e-3 / (reps * 2)
-    kern = f"k_line_zebra<{'float' if f32 else 'double'}>" + (" 5-point" if five else "")
-    elems = 10.0 if five else 14.0
+    rows = f32 and g.nx - 2 <= 4096  # factored as they are solved: E and diag instead of five factor arrays
+    kern = ("k_line_row" if rows else f"k_line_zebra<{'float' if f32 else 'double'}>") + (" 5-point" if five else "")
+    elems = (10.0 if five else 14.0) - (3.0 if rows else 0.0)
     bytes_per_launch = elems * esz * g.nx * g.nyr / 2
     ach = bytes_per_launch / per_launch_s / 1e9
     return _hbm_roof(kern, ach, per_launch_s, g, elements_per_node_and_sweep=elems)
