@@ -111,7 +111,8 @@ __global__ void __launch_bounds__(kRRX* kRRY)
 // couplings and from all rows of x.  One thread per coarse node computes r(2I) and r(2I+1)
 // of row 2J; r(2I-1) is its left neighbour's r(2I+1), handed over in shared memory (the
 // block's first thread computes the one left of the block).  Summation order as in
-// k_resid_restrict with the odd-row terms zero.
+// k_resid_restrict with the odd-row terms zero.  xH (nullable): a coarse iterate whose boundary
+// nodes are zeroed.
 template <typename T>
 __global__ void __launch_bounds__(kREven) k_resid_restrict_even(Lvl<T> L, const T* __restrict__ x,
                                                                 const T* __restrict__ b, T* __restrict__ bH,
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(kREven) k_resid_restrict_even(Lvl<T> L, const 
   const bool unk = (I >= 1 && I <= nxc - 2) && (L.periodic || (J >= 1 && J <= nyc - 2));
   const size_t K = (size_t)J * pitchc + I;
   bH[K] = unk ? (T(4) * r0 + T(2) * (rodd[threadIdx.x] + r1)) * T(0.0625) : T(0);
-  if (xH) xH[K] = T(0);
+  if (xH && !unk) xH[K] = T(0);
 }
 
 // x += P eH (bilinear: injection at coincident nodes, 1/2 on edges, 1/4 at centres).  A thread corrects

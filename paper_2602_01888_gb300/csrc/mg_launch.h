@@ -129,7 +129,8 @@ template <typename T>
 cudaError_t launch_resid_restrict(const Op<T>& A, const T* phi, const T* b, T* bH, T* phiH,
                                   int pitch_c, const int* skip, cudaStream_t s);
 // The same after a pre-smoothing whose last half-sweep solved every odd row exactly (zebra
-// x-line): the odd rows' residual is taken as zero and only the even rows' is computed.
+// x-line): the odd rows' residual is taken as zero and only the even rows' is computed.  phiH
+// (nullable): its boundary nodes are zeroed (a level smoothed from zero reads no other ones).
 template <typename T>
 cudaError_t launch_resid_restrict_even(const Op<T>& A, const T* phi, const T* b, T* bH, T* phiH,
                                        int pitch_c, const int* skip, cudaStream_t s);

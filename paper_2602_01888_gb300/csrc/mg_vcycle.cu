@@ -171,10 +171,12 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
       const int zero = l == 0 ? (x0_zero && zs) : zs;
       if ((e = launch_line_smooth(V.A[l], V.lf[l], cur[l], V.b[l], nu1, 0, skip, s, (const T*)nullptr, 0, zero)))
         return e;
-      // without pre-smoothing a coarse level's iterate is read, so it is cleared here (the tail
-      // kernel starts from zero by itself).  After pre-smoothing, whose last half-sweep solved
-      // the odd rows, only the even rows' residual is restricted (launch_resid_restrict_even).
-      T* const xc = zs || l + 1 == t ? nullptr : cur[l + 1];
+      // A coarse level starts from zero, boundary nodes included, whatever its array holds.  After
+      // pre-smoothing, whose last half-sweep solved the odd rows, only the even rows' residual is
+      // restricted (launch_resid_restrict_even) and only the next level's boundary is cleared: its
+      // first half-sweep or the coarsest solve writes every unknown that is read later.  Without
+      // pre-smoothing its whole iterate is cleared.  The tail kernel starts from zero by itself.
+      T* const xc = l + 1 == t && t < L - 1 ? nullptr : cur[l + 1];
       if ((e = zs ? launch_resid_restrict_even(V.A[l], cur[l], V.b[l], V.b[l + 1], xc, V.A[l + 1].pitch, skip, s)
                   : launch_resid_restrict(V.A[l], cur[l], V.b[l], V.b[l + 1], xc, V.A[l + 1].pitch, skip, s)))
         return e;
