@@ -290,18 +290,19 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
       alt[l] = tmp;
     };
     if (kind == SK_BLOCK) {  // passes of two sweeps, an odd one first
+      // the fused restriction takes levels whose sides are 2 m + 1, as every exact hierarchy's are
+      const bool fuse = bH && (V.A[l].nx - 1) % 2 == 0 && (V.A[l].ny - 1) % 2 == 0;
       for (int left = sweeps; left > 0;) {
         const int ns = left % 2 ? 1 : 2;
         const bool first = left == sweeps, last = left == ns;
         err = launch_smooth_block<T>(V.A[l], first && zero ? nullptr : cur[l], alt[l], V.b[l], ns, rev,
-                                     first ? eH : nullptr, last ? bH : nullptr, pc, skip, s);
+                                     first ? eH : nullptr, last && fuse ? bH : nullptr, pc, skip, s);
         if (err) return err;
         swap_cur();
         left -= ns;
       }
-      return xH ? clear(l + 1) : cudaSuccess;
-    }
-    if (kind == SK_MARCH) {
+      if (fuse) return xH ? clear(l + 1) : cudaSuccess;
+    } else if (kind == SK_MARCH) {
       for (int k = 0; k < sweeps / march_sweeps<T>(var); ++k) {
         err = launch_smooth_march<T>(V.A[l], cur[l], alt[l], V.b[l], rev, k == 0 ? eH : nullptr, pc, skip, s,
                                      var);
