@@ -340,8 +340,13 @@ static int blk_sms() {
 template <typename T>
 bool block_can(const Op<T>& A, const T* xin, const T* xout, const T* b) {
   const uintptr_t all = (uintptr_t)xin | (uintptr_t)xout | (uintptr_t)b | (uintptr_t)A.cE | (uintptr_t)A.cN |
-                        (uintptr_t)A.cNE | (uintptr_t)A.cNW | (uintptr_t)A.diag | (uintptr_t)A.dinv;
+                        (uintptr_t)A.cNE | (uintptr_t)A.cNW | (uintptr_t)A.dinv;
   return A.pitch % (16 / (int)sizeof(T)) == 0 && all % 16 == 0 && !(A.periodic && (A.ny - 1) % 2);
+}
+
+template <typename T>
+bool block_can_restrict(const Op<T>& A) {
+  return (uintptr_t)A.diag % 16 == 0 && (A.nx - 1) % 2 == 0 && (A.ny - 1) % 2 == 0;
 }
 
 template <typename T, int NS, int TX, int TY, bool RR>
@@ -379,7 +384,7 @@ static cudaError_t block_impl(const Op<T>& A, const T* xin, T* xout, const T* b,
 template <typename T>
 cudaError_t launch_smooth_block(const Op<T>& A, const T* xin, T* xout, const T* b, int ns, int rev, const T* eH, T* bH,
                                 int pitch_c, const int* skip, cudaStream_t s) {
-  if (xin == xout || !block_can(A, xin, xout, b) || (bH && (rev || eH || (A.nx - 1) % 2 || (A.ny - 1) % 2)))
+  if (xin == xout || !block_can(A, xin, xout, b) || (bH && (rev || eH || !block_can_restrict(A))))
     return cudaErrorInvalidValue;
   if (ns != 1 && ns != 2) return cudaErrorInvalidValue;
   const int nyr = rows_stored(A.ny, A.periodic);
@@ -406,6 +411,7 @@ cudaError_t launch_smooth_block(const Op<T>& A, const T* xin, T* xout, const T* 
 
 #define MG_BLOCK_INST(T)                                                                                             \
   template bool block_can<T>(const Op<T>&, const T*, const T*, const T*);                                            \
+  template bool block_can_restrict<T>(const Op<T>&);                                                                 \
   template cudaError_t launch_smooth_block<T>(const Op<T>&, const T*, T*, const T*, int, int, const T*, T*, int,     \
                                               const int*, cudaStream_t);
 MG_BLOCK_INST(float)

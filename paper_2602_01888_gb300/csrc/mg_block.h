@@ -16,10 +16,14 @@ constexpr int block_tile_width() {
 // aligned, and an even row count on a periodic level.
 template <typename T>
 bool block_can(const Op<T>& A, const T* xin, const T* xout, const T* b);
+// Whether it can also restrict the residual: sides of 2 m + 1, as in every exact hierarchy, and the
+// diagonal (which smoothing alone does not read) 16-byte aligned.
+template <typename T>
+bool block_can_restrict(const Op<T>& A);
 
 // xout = ns four-colour Gauss-Seidel sweeps of (xin [+ P eH]) in forward (rev = 0) or reversed
 // colour order; xin != xout.  xin == nullptr: a zero iterate.  bH (nullable; rev = 0, eH
-// nullptr, even nx - 1 and ny - 1): also the full weighting of b - A xout at the coarse nodes (0
+// nullptr, block_can_restrict): also the full weighting of b - A xout at the coarse nodes (0
 // on the coarse boundary ring; row pitch pitch_c).  pitch_c is eH's row pitch otherwise.
 template <typename T>
 cudaError_t launch_smooth_block(const Op<T>& A, const T* xin, T* xout, const T* b, int ns, int rev, const T* eH, T* bH,

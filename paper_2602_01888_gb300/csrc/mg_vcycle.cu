@@ -290,8 +290,7 @@ cudaError_t emit_vcycle(const VLevels<T>& V, int smoother, int nu1, int nu2, dou
       alt[l] = tmp;
     };
     if (kind == SK_BLOCK) {  // passes of two sweeps, an odd one first
-      // the fused restriction takes levels whose sides are 2 m + 1, as every exact hierarchy's are
-      const bool fuse = bH && (V.A[l].nx - 1) % 2 == 0 && (V.A[l].ny - 1) % 2 == 0;
+      const bool fuse = bH && block_can_restrict(V.A[l]);
       for (int left = sweeps; left > 0;) {
         const int ns = left % 2 ? 1 : 2;
         const bool first = left == sweeps, last = left == ns;
