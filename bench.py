@@ -492,6 +492,7 @@ def measure_smoother(mg, torch, inst, prec, reps=20, smoother="gs4", family=None
     fam, shape = parse_choice(family)
     if fam is None:  # untuned: the size rule of the cycle
         fam = "marching" if f32 or g.nx * g.nyr >= MARCH_NODES else "colour"
+        shape = (52, 0, 2) if f32 else None  # the register blocks
     if fam in ("pipelined", "fused", "marching"):
         return _measure_variant(mg, torch, g, st, x, z(dt), b, f32, s, reps, fam, shape)
 
@@ -722,8 +723,9 @@ def run_kernel_only(args):
         fac = torch.zeros(mg.lib().mgk_line_factor_elems(n, g.ny, 0), dtype=dt, device="cuda")
         mg.mgk(f"mgk_line_factor_{sfx}", C.byref(st), fac.data_ptr(), s)
 
-    # the family's default variant unless --variant picks another (fused: FP64 32x32/1, FP32 64x24/2)
-    var = args.variant if args.variant >= 0 else (5 if args.kernel.startswith("fused") and not f64 else 0)
+    # the family's default variant unless --variant picks another (fused: FP64 32x32/1, FP32 64x24/2;
+    # march: FP32 the register blocks)
+    var = args.variant if args.variant >= 0 else (5 if args.kernel.startswith(("fused", "march")) and not f64 else 0)
 
     def once():
         if args.kernel.startswith("line"):  # one zebra sweep: two launches of k_line_zebra

@@ -44,8 +44,8 @@ namespace mg {
 template <typename T, int CFG>
 struct MarchGeom;
 
-// Geometries, by precision and configuration number (FP32: configuration 0 is the default;
-// FP64: configuration 3, see f64_cfg).  C loaded columns (C/2 per parity), HX halo columns and HY = 4 NS halo rows each
+// Geometries, by precision and configuration number (variants and defaults: kMarchCfgF32,
+// kMarchCfgF64).  C loaded columns (C/2 per parity), HX halo columns and HY = 4 NS halo rows each
 // side, R ring rows, D rows in flight, LCH 16-byte chunks per loader thread and row.
 //
 // FP32 0: two sweeps a pass.  1024 threads: 512 compute (4 active phases x 128 nodes), 448
@@ -562,9 +562,11 @@ __global__ void __launch_bounds__(MarchGeom<T, CFG>::THREADS, MarchGeom<T, CFG>:
 }
 
 // Variants: kMarchCfg gives the configuration of MarchGeom, or -2 for a register-block pass of two
-// sweeps (k_block.cu).  Variant 0 is each precision's default: FP32 the register blocks, FP64
-// configuration 3.
-constexpr int kMarchCfgF32[] = {-2, 0, 1, 2, 3, 4};
+// sweeps (k_block.cu).  A variant keeps its number (callers may store one), so new ones come last.
+// Defaults: FP32 the register blocks; FP64 configuration 3, measured the fastest at 2049^2-8193^2
+// (1.46 ms a sweep at 8193^2 against 1.69 for configuration 2 and 2.26 for configuration 0, whose
+// four compute warps leave the FP64 pipe waiting on their dependent FMA chains).
+constexpr int kMarchCfgF32[] = {0, 1, 2, 3, 4, -2};
 constexpr int kMarchCfgF64[] = {3, 1, 2, 0, -2};
 
 template <typename T>
@@ -574,7 +576,7 @@ int march_variants() {
 
 template <typename T>
 static int march_cfg_of(int v) {
-  if (v < 0 || v >= march_variants<T>()) v = 0;
+  if (v < 0 || v >= march_variants<T>()) return sizeof(T) == 8 ? 3 : -2;
   return sizeof(T) == 8 ? kMarchCfgF64[v] : kMarchCfgF32[v];
 }
 
