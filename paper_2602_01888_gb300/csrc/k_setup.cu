@@ -71,11 +71,11 @@ __global__ void __launch_bounds__(256) k_eps_sine_warp(double p0, int nx, int ny
 
 // Polar map (Eq. 29), the general formula with what depends on one coordinate taken out of the node:
 // the row's sum of squares, and 1 / x for the division.  det J = x (cos^2 + sin^2) is x but for
-// rounding, so one Newton step from 1 / x gives 1 / det to one rounding.  The closed form (D = x,
-// eps_xx = s x, eps_yy = s / x) would be cheaper still, but its rounding is the same at every node of
-// a circle and adds up in the row sums of the operator: at 8193^2 it moves the solution by 3e-10.
-// Ten FP64 operations a node bound it: 8193 x 8192 1.43 ms, 2.60 ms with the division and the sums at
-// every node.
+// rounding, so the quotient eps' / x corrected by its residual against det J is eps' / det J to one
+// rounding.  The closed form (D = x, eps_xx = s x, eps_yy = s / x) would be cheaper still, but its
+// rounding is the same at every node of a circle and adds up in the row sums of the operator: at
+// 8193^2 it moves the solution by 3e-10.  Ten FP64 operations a node bound it: 8193 x 8192 1.43 ms (1.54
+// with a material), 2.60 ms with the division and the sums at every node.
 __global__ void __launch_bounds__(256) k_eps_polar(int nx, int nyr, double x0, double y0, double hx, double hy,
                                                    const double* __restrict__ eps, int pitch,
                                                    double* __restrict__ D, double* __restrict__ exx,
@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(256) k_eps_polar(int nx, int nyr, double x0, d
     if (folds(det)) atomicOr(folded, 1);
     const size_t k = (size_t)j * pitch + i;
     D[k] = det;
-    double sd = fma(rx, fma(-det, rx, 1.0), rx);
-    if (eps) sd *= eps[k];
+    const double m = eps ? eps[k] : 1.0, q = m * rx;
+    const double sd = fma(rx, fma(-det, q, m), q);
     exx[k] = sd * (d * d + b * b);  // Eq. 12
     exy[k] = 0.0;                   // Eq. 13 vanishes identically
     eyy[k] = sd * rowv[2][ly];      // Eq. 15
