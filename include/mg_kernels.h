@@ -45,7 +45,8 @@ typedef struct {
  * (device int) is set to 1 where D <= 0 and left unchanged elsewhere.  For a map without
  * cross term (mg_map_five_point of mg.h: identity, polar, sinh, shear-free affine) eps_xy
  * is written as exactly 0, which Eq. 13 is for it (the general formula would leave rounding
- * residue); D, eps_xx and eps_yy always come from the general formula.
+ * residue).  D, eps_xx and eps_yy of the identity, sinh and affine maps are products of a factor
+ * of x and a factor of y; the other maps' come from the general formula.
  */
 int mgk_eps_analytic(int kind, const double *params4, int nx, int ny, int periodic, double x0,
                      double y0, double hx, double hy, const double *eps_phys, int pitch, double *D,
@@ -64,7 +65,8 @@ int mgk_eps_grid(int nx, int ny, int periodic, double hx, double hy, const doubl
  * Fine-level operator A = -L_h from nodal eps (symmetric conservative form of the
  * Eq. 18 stencil): E/N couplings -(face mean of eps_xx / eps_yy)/h^2, corner couplings
  * from (Dx E Dy + Dy E Dx) with E = diag(eps_xy), diagonal = -(sum of the 8 couplings)
- * at unknowns, 1 at Dirichlet nodes.  Couplings missing at the grid edge are 0.  With
+ * at unknowns (formed from the E, W, N and S ones, since the corner couplings of a node cancel
+ * exactly before they are rounded), 1 at Dirichlet nodes.  Couplings missing at the grid edge are 0.  With
  * A->five_point set, eps_xy is taken as zero (it is not read) and cNE, cNW are written as 0.
  */
 int mgk_assemble(const mgk_op_f64 *A, double hx, double hy, const double *exx, const double *exy,
@@ -200,13 +202,14 @@ int mgk_smooth_pipe_f32(const mgk_op_f32 *A, const float *xin, float *xout, cons
                         int reverse, const float *eH, int pitch_c, int *err, void *stream);
 int mgk_pipe_sweeps(int f32);
 
-/* Row-marching variant for large levels: xout = mgk_march_sweeps() (FP32) or
- * mgk_march_sweeps_f64() (FP64) four-colour Gauss-Seidel sweeps (Sec. 2.1, omega = 1;
- * reverse = 1 reverses the colour order) of xin [+ P eH] (Eq. 24) in one pass over the
- * level.  Each CTA streams a strip of columns upward through a ring of rows in shared
- * memory, so every array is read about once.  Same result as the per-colour kernels
+/* One pass over a level: xout = mgk_march_sweeps() (FP32) or mgk_march_sweeps_f64() (FP64)
+ * four-colour Gauss-Seidel sweeps (Sec. 2.1, omega = 1; reverse = 1 reverses the colour order) of
+ * xin [+ P eH] (Eq. 24), every array read about once.  FP64: each CTA streams a strip of columns
+ * upward through a ring of rows in shared memory.  FP32: tiles whose couplings stay in registers
+ * (the strips are variants of mgk_smooth_variant_f32).  Same result as the per-colour kernels
  * (identical operations in the same order per node).  Needs xin != xout, 16-byte aligned
- * arrays and a pitch that keeps rows 16-byte aligned (else returns 1); 4 on a CUDA error. */
+ * arrays (the diagonal, which smoothing does not read, excepted) and a pitch that keeps rows
+ * 16-byte aligned (else returns 1); 4 on a CUDA error. */
 int mgk_smooth_march_f32(const mgk_op_f32 *A, const float *xin, float *xout, const float *b,
                          int reverse, const float *eH, int pitch_c, void *stream);
 int mgk_smooth_march_f64(const mgk_op_f64 *A, const double *xin, double *xout, const double *b,
@@ -217,10 +220,11 @@ int mgk_march_sweeps_f64(void);
 /* Shapes the autotuner chooses among (mg_autotune).  family: 2 fused tiles, 3 pipelined
  * tiles, 4 row marching (the mg_tune_entry.choice codes).  mgk_smooth_variant_info gives
  * variant `variant` of a family in FP32 (f32 = 1) or FP64: owned tile tile_x x tile_y
- * (marching: tile_x owned strip columns, tile_y 0) and sweeps per launch; returns 1 past the
- * last variant.  mgk_smooth_variant_* runs one launch of that variant exactly as the
- * mgk_smooth_fused_* / mgk_smooth_pipe_* / mgk_smooth_march_* entry points run their default
- * one (same arguments and requirements; err is used by the pipelined tiles only). */
+ * (marching: tile_x owned columns of a strip, or of a register-block tile for the last variant,
+ * tile_y 0) and sweeps per launch; returns 1 past the last variant.  A variant keeps its number.
+ * mgk_smooth_variant_* runs one launch of that variant exactly as the mgk_smooth_fused_* /
+ * mgk_smooth_pipe_* / mgk_smooth_march_* entry points run their default one (same arguments and
+ * requirements; err is used by the pipelined tiles only). */
 int mgk_smooth_variant_info(int f32, int family, int variant, int *tile_x, int *tile_y, int *sweeps);
 int mgk_smooth_variant_f64(const mgk_op_f64 *A, int family, int variant, const double *xin, double *xout,
                            const double *b, int reverse, const double *eH, int pitch_c, int *err,
@@ -234,13 +238,14 @@ int mgk_smooth_variant_f32(const mgk_op_f32 *A, int family, int variant, const f
  * half-sweep of parity p solves, for every row j with j mod 2 == p, the tridiagonal system
  * of the row's unknowns (diagonal, W and E couplings) with the couplings to rows j-1 and
  * j+1 (N, S, NE, NW, SE, SW) and to the row's two Dirichlet end nodes moved to the
- * right-hand side; rows of one parity are independent.  The row systems are solved by
- * cyclic reduction (row length nx - 2 padded to a power of two) with factors that depend
- * on A only:
+ * right-hand side; rows of one parity are independent.  The row systems are solved directly, with
+ * stored factors that depend on A only (cyclic reduction over the row length nx - 2 padded to a
+ * power of two; in FP64 rows padded to 2048 or 4096 by partition into segments), or, in FP32 for
+ * rows of up to 4096 unknowns, factored as they are solved from A's E couplings and diagonal:
  *   mgk_line_factor_elems(nx, ny, periodic): elements (of the operator's precision) that
  *     the factors of an nx x ny level take; 0 for sizes below 3;
  *   mgk_line_factor_*: fills `factors` for every row of A; call it again when A changes
- *     (FP32 rows of up to 4096 unknowns are factored as they are solved: nothing is written);
+ *     (nothing is written for rows that are factored as they are solved);
  *   mgk_line_rows_*: one half-sweep of parity 0 or 1, phi updated in place;
  *   mgk_line_smooth_*: `sweeps` sweeps, each parity 0 then 1 (reverse != 0: 1 then 0).
  * Rows of up to 8192 unknowns in FP64 and 16384 in FP32 (shared-memory bound); longer

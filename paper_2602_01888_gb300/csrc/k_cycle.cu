@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kREven) k_resid_restrict_even(Lvl<T> L, const 
 }
 
 // x += P eH (bilinear: injection at coincident nodes, 1/2 on edges, 1/4 at centres).  A thread corrects
-// the 2 x 2 fine nodes up and right of a coarse node: eight operations for the four, without the
+// the 2 x 2 fine nodes up and right of a coarse node: nine operations for the four, without the
 // divergence of one thread a node (in FP64 five issue slots a node, on the pipe that bounds it):
 // FP64 1025^2 14.9 -> 9.4 us.  VEC: pairs of columns in one access.
 template <typename T, bool VEC>

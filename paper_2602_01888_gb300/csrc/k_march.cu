@@ -19,9 +19,9 @@
 // columns at distance > ph from the loaded edge; after 4 NS phases the owned rows and
 // columns hold exactly the result of NS sequential sweeps.
 //
-// Geometry per precision: FP32 two sweeps a pass on 256-column strips, FP64 one sweep a
-// pass on 128-column strips by default; the other depth of each is a variant the autotuner
-// may pick (MarchGeom below).
+// Geometry per precision (MarchGeom below): FP64 one sweep a pass on 128-column strips by default,
+// other depths and widths as variants the autotuner may pick; FP32 variants only, its default being
+// the register blocks (k_block.cu).
 //
 // The threads of a CTA have one role each, in whole warps: compute threads run the
 // phases; loader threads request rows D steps ahead with asynchronous 16-byte copies into

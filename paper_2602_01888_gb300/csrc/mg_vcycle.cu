@@ -61,8 +61,10 @@ int line_tail_nodes() {
   return v;
 }
 
-// Levels with more nodes than this use the per-colour smoothing kernels (four launches
-// a sweep); smaller levels above the tail use the fused tile kernel.
+// Among the levels above the tail that the register blocks do not take (FP64 levels of more than
+// block_nodes_f64() nodes; rows or arrays off 16-byte boundaries, an odd period in y): more nodes than
+// this use the per-colour smoothing kernels (four launches a sweep; FP32 of aligned rows the pipelined
+// tiles), fewer the fused tile kernel.
 template <typename T>
 int colour_nodes() {
   static int v = -1;
@@ -88,8 +90,8 @@ inline long long block_nodes_f64() {
   return v;
 }
 
-// Levels with at least this many nodes use the row-marching smoother; below it the grid has
-// too few strips and segments to fill the GPU.
+// FP64 levels with at least this many nodes use the row-marching smoother; below it the grid has too
+// few strips and segments to fill the GPU.  (FP32 levels never do: see the rule below.)
 inline long long march_nodes() {
   static long long v = -1;
   if (v < 0) {
