@@ -144,9 +144,11 @@ __global__ void __launch_bounds__(kREven) k_resid_restrict_even(Lvl<T> L, const 
 
 // x += P eH (bilinear: injection at coincident nodes, 1/2 on edges, 1/4 at centres).  A thread corrects
 // the 2 x 2 fine nodes up and right of a coarse node: nine operations for the four, without the
-// divergence of one thread a node (in FP64 five issue slots a node, on the pipe that bounds it):
-// FP64 1025^2 14.9 -> 9.4 us.  VEC: pairs of columns in one access.
-template <typename T, bool VEC>
+// divergence of one thread a node (in FP64 five issue slots a node, on the pipe that bounds it): FP64
+// 129^2 2.15 -> 2.25 us, 513^2 4.8 -> 3.0, 1025^2 12.3 -> 6.6, 4097^2 164 -> 68; FP32 129^2 1.95 -> 1.9,
+// 4097^2 63.6 -> 18.8 (graph replays).  Two columns in one access, where rows allow it, were slower
+// (FP32 4097^2 23.0, 129^2 2.4): the branch that keeps them apart at the edges costs more.
+template <typename T>
 __global__ void __launch_bounds__(256) k_prolong_add(Lvl<T> L, T* __restrict__ x,
                                                      const T* __restrict__ eH, int nxc, int nyrc,
                                                      int pitchc, const int* __restrict__ skip) {
@@ -161,21 +163,14 @@ __global__ void __launch_bounds__(256) k_prolong_add(Lvl<T> L, T* __restrict__ x
   const T eb = e ? eH[a + 1] : T(0), ed = e ? eH[c + 1] : T(0);
   const T lo = ea + eb, le = ea + ec, all = lo + (ec + ed);
   T* const p = x + (size_t)j * L.pitch + i;
-  auto row = [&](T* q, int jj, T d0, T h, T w) {  // q[0] += d0, q[1] += w h at the unknowns of row jj
-    const bool u0 = is_unknown(L, i, jj), u1 = is_unknown(L, i + 1, jj);
-    if (VEC && u0 && u1) {
-      using P = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
-      P v = *reinterpret_cast<P*>(q);
-      v.x += d0;
-      v.y = fma(w, h, v.y);
-      *reinterpret_cast<P*>(q) = v;
-    } else {
-      if (u0) q[0] += d0;
-      if (u1) q[1] = fma(w, h, q[1]);
-    }
-  };
-  row(p, j, ea, lo, T(0.5));
-  row(p + L.pitch, j + 1, T(0.5) * le, all, T(0.25));
+  T* const q = p + L.pitch;
+  const bool pa = is_unknown(L, i, j), pb = is_unknown(L, i + 1, j), qa = is_unknown(L, i, j + 1), qb = is_unknown(L, i + 1, j + 1);
+  // all four loads before the first store (which they could not pass)
+  const T a0 = pa ? p[0] : T(0), b0 = pb ? p[1] : T(0), a1 = qa ? q[0] : T(0), b1 = qb ? q[1] : T(0);
+  if (pa) p[0] = a0 + ea;
+  if (pb) p[1] = fma(T(0.5), lo, b0);
+  if (qa) q[0] = fma(T(0.5), le, a1);
+  if (qb) q[1] = fma(T(0.25), all, b1);
 }
 
 // x = inv * b at the coarsest unknowns (lexicographic, i fastest), one CTA.
@@ -293,10 +288,7 @@ cudaError_t launch_prolong_add(const Op<T>& A, T* phi, const T* eH, int pitch_c,
   const int nxc = (A.nx - 1) / 2 + 1, nyrc = rows_stored((A.ny - 1) / 2 + 1, A.periodic);
   dim3 bl(32, 8);
   const dim3 g = g2(nxc, nyrc, bl);
-  if (A.pitch % 2 == 0 && (uintptr_t)phi % (2 * sizeof(T)) == 0)
-    k_prolong_add<T, true><<<g, bl, 0, s>>>(L, phi, eH, nxc, nyrc, pitch_c, skip);
-  else
-    k_prolong_add<T, false><<<g, bl, 0, s>>>(L, phi, eH, nxc, nyrc, pitch_c, skip);
+  k_prolong_add<T><<<g, bl, 0, s>>>(L, phi, eH, nxc, nyrc, pitch_c, skip);
   return cudaGetLastError();
 }
 
