@@ -298,7 +298,7 @@ __global__ void k_assemble_diag(int nx, int ny, int nyr, int periodic, int pitch
 // One pass over the finest level: the couplings of k_assemble_couplings, the diagonal, its reciprocal
 // (dinv when given) and, when fE is given, the FP32 copy of k_op_to_f32 with the reciprocal of the FP32
 // diagonal (pitch pf).  A warp covers 32 columns, of which it owns the inner 30, and marches down
-// kAsmRows rows: every tensor value is loaded once (shuffles and the row before give the
+// a strip of rows: every tensor value is loaded once (shuffles and the row before give the
 // neighbours').  A coupling is rounded like the separate kernel's: -(1/2)(a + b) / h^2 is the sum times
 // the exact constant -(1/2) / h^2 (halving is exact), one rounding per operation (__dadd_rn,
 // __dmul_rn: no contracted multiply-add), so the couplings are bitwise those of the separate kernels.
@@ -308,20 +308,19 @@ __global__ void k_assemble_diag(int nx, int ny, int nyr, int periodic, int pitch
 // the kernels that have no 5-point form.  Bound by the FP64 pipe: 11 operations a node (FIVE: 7) and
 // the five of dinv's reciprocal.  9-point 2049^2 157 us, 197 us with the two separate kernels; 5-point
 // 8193^2 with the FP32 copy 1.33 -> 1.22 ms (every first lane computed its W coupling, predicated).
-constexpr int kAsmRows = 8;
 constexpr int kAsmCols = 30;
 
 template <bool FIVE>
 __global__ void __launch_bounds__(256) k_assemble_pass(int nx, int ny, int nyr, int periodic, int pitch, double mx,
                                                        double my, double mxy, const double* __restrict__ exx,
                                                        const double* __restrict__ exy,
-                                                       const double* __restrict__ eyy, double* cE, double* cN,
+                                                       const double* __restrict__ eyy, int rows, double* cE, double* cN,
                                                        double* cNE, double* cNW, double* diag, double* dinv, int pf,
                                                        float* fE, float* fN, float* fNE, float* fNW, float* fdiag,
                                                        float* fdinv) {
   const int lane = threadIdx.x;
   const int i = blockIdx.x * kAsmCols + lane - 1;
-  const int jb = (blockIdx.y * blockDim.y + threadIdx.y) * kAsmRows;
+  const int jb = (blockIdx.y * blockDim.y + threadIdx.y) * rows;
   if (jb >= nyr) return;  // one strip per warp
   const bool col = i >= 0 && i < nx, own = col && lane >= 1 && lane <= kAsmCols, has_e = i + 1 <= nx - 1;
   auto get = [&](const double* __restrict__ f, int j) { return col ? f[(size_t)j * pitch + i] : 0.0; };
@@ -343,7 +342,7 @@ __global__ void __launch_bounds__(256) k_assemble_pass(int nx, int ny, int nyr, 
     const int jm = jb == 0 ? nyr - 1 : jb - 1;
     ns = __dmul_rn(__dadd_rn(get(eyy, jm), y), my);
   }
-  for (int r = 0; r < kAsmRows; ++r) {
+  for (int r = 0; r < rows; ++r) {
     const int j = jb + r;
     if (j >= nyr) break;
     const int ju = (j + 1 == nyr) ? 0 : j + 1;
@@ -759,10 +758,17 @@ template <bool FIVE>
 static cudaError_t assemble_pass(const OpF64& A, const OpF32* B, double hx, double hy, const double* exx,
                                  const double* exy, const double* eyy, cudaStream_t s, bool dinv) {
   const int nyr = rows_stored(A.ny, A.periodic);
-  dim3 b(32, 8), g((A.nx + kAsmCols - 1) / kAsmCols, (nyr + 8 * kAsmRows - 1) / (8 * kAsmRows));
+  // strips of eight rows (one row is read twice a strip); shorter ones on grids too small to hide a
+  // strip's chain of loads (9-point, us by rows 1 / 2 / 8, two separate kernels: 129^2 3.0 / 4.4 / 12.7,
+  // 4.7; 385^2 8.5 / 9.5 / 12.9, 11.5; 769^2 25.4 / 25.4 / 32.0, 31.0; 1025^2 43.5 / 41.4 / 42.8, 51.3;
+  // 2049^2 165 / 158 / 154, 195)
+  const int gx = (A.nx + kAsmCols - 1) / kAsmCols;
+  const long long warps = (long long)gx * nyr;  // of one row each
+  const int rows = warps <= 40 * 152 ? 1 : warps <= 240 * 152 ? 2 : 8;
+  dim3 b(32, 8), g(gx, (nyr + 8 * rows - 1) / (8 * rows));
   k_assemble_pass<FIVE><<<g, b, 0, s>>>(
       A.nx, A.ny, nyr, A.periodic, A.pitch, -0.5 * (1.0 / (hx * hx)), -0.5 * (1.0 / (hy * hy)), 1.0 / (4.0 * hx * hy), exx,
-      exy, eyy, A.cE, A.cN, A.cNE, A.cNW, A.diag, dinv ? A.dinv : nullptr, B ? B->pitch : 0, B ? B->cE : nullptr,
+      exy, eyy, rows, A.cE, A.cN, A.cNE, A.cNW, A.diag, dinv ? A.dinv : nullptr, B ? B->pitch : 0, B ? B->cE : nullptr,
       B ? B->cN : nullptr, B ? B->cNE : nullptr, B ? B->cNW : nullptr, B ? B->diag : nullptr, B ? B->dinv : nullptr);
   return cudaGetLastError();
 }
