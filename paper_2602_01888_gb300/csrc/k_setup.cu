@@ -518,7 +518,7 @@ __global__ void k_galerkin(Lvl<T> F, int nxc, int nyc, int nyrc, int pitchc, T* 
 // and the second combines the rows 2J - 1, 2J, 2J + 1 the same way.  A warp holds 32 coarse columns,
 // of which it owns the inner 30 (the lanes beside supply E's and NW's missing halves), and marches
 // up a strip of coarse rows, so each fine row is collapsed once.  Pairs of columns are loaded as one
-// vector.  FIVE: zero NE / NW, whose terms vanish exactly (46 operations).  Bound by the FP64 pipe
+// vector.  FIVE: zero NE / NW, whose terms vanish exactly (42 operations).  Bound by the FP64 pipe
 // (81% busy): 2049^2 -> 1025^2 -> 513^2 220 us, 292 us with k_galerkin.  The sums are ordered so that
 // large terms cancel before small ones are added.  Rms errors against exact sums as fractions of the
 // direct product's (which stay below 8e-17 of the largest coupling off the diagonal and 2.3e-16 on it),
@@ -543,6 +543,7 @@ __global__ void __launch_bounds__(128, 5) k_galerkin_rows(Lvl<double> F, int nxc
   const bool col = I >= 0 && I < nxc, own = col && lane >= 1 && lane <= kGalCols;
   auto left = [](double v) { return __shfl_up_sync(0xffffffffu, v, 1); };
   auto right = [](double v) { return __shfl_down_sync(0xffffffffu, v, 1); };
+  constexpr double hu = FIVE ? 0.125 : 0.5;
   auto row = [&](int j) -> GalRow {  // j wrapped or clamped into the grid by the caller
     const size_t k = (size_t)j * F.pitch + 2 * I;
     const double2 z = make_double2(0.0, 0.0);
@@ -553,9 +554,9 @@ __global__ void __launch_bounds__(128, 5) k_galerkin_rows(Lvl<double> F, int nxc
     g.h0 = fma(0.25, dl + d.y, (d.x + e.x) + el);
     g.h1 = fma(0.5, e.x, fma(0.5, e.y, 0.25 * d.y));
     g.u0 = fma(0.25, nl + n.y, n.x);
-    if (FIVE) {
-      g.u1 = 0.25 * n.y;
-      g.um = 0.25 * nl;
+    if (FIVE) {  // four times u1 and um: hu takes the factor
+      g.u1 = n.y;
+      g.um = nl;
     } else {
       const double2 ne = get(F.cNE), nw = get(F.cNW);
       const double nel = left(ne.y), nwl = left(nw.y);
@@ -577,10 +578,10 @@ __global__ void __launch_bounds__(128, 5) k_galerkin_rows(Lvl<double> F, int nxc
       double vE = 0.0, vN = 0.0, vNE = 0.0, vNW = 0.0, vd = 1.0;
       if (unk) {
         vd = 0.25 * fma(0.25, p.h0, fma(0.25, n.h0, c.h0 + (p.u0 + c.u0)));
-        vE = 0.25 * fma(0.25, p.h1 + n.h1, fma(0.5, s_um, fma(0.5, c.u1, fma(0.5, p.u1, c.h1))));
+        vE = 0.25 * fma(0.25, p.h1 + n.h1, fma(hu, s_um, fma(hu, c.u1, fma(hu, p.u1, c.h1))));
         vN = 0.25 * fma(0.5, c.u0, fma(0.5, n.u0, 0.25 * n.h0));
-        vNE = 0.25 * fma(0.5, c.u1, fma(0.5, n.u1, 0.25 * n.h1));
-        vNW = 0.25 * fma(0.5, c.um, fma(0.5, n.um, 0.25 * h1l));
+        vNE = 0.25 * fma(hu, c.u1, fma(hu, n.u1, 0.25 * n.h1));
+        vNW = 0.25 * fma(hu, c.um, fma(hu, n.um, 0.25 * h1l));
       }
       diag[K] = vd;
       dinv[K] = unk ? 1.0 / vd : 1.0;
@@ -815,10 +816,13 @@ cudaError_t launch_galerkin(const Op<T>& F, const Op<T>& C, cudaStream_t s) {
   if constexpr (sizeof(T) == 8) {
     const uintptr_t all = (uintptr_t)F.cE | (uintptr_t)F.cN | (uintptr_t)F.cNE | (uintptr_t)F.cNW | (uintptr_t)F.diag;
     if (F.pitch % 2 == 0 && all % 16 == 0) {  // rows readable in pairs of columns
-      // strips of eight coarse rows (one more fine row collapsed per strip: 6%), shorter on small
-      // levels, whose few warps would leave SMs idle
+      // strips of eight coarse rows (one more fine row collapsed per strip: 6%), shorter on small levels,
+      // whose few warps would leave SMs idle and wait for a strip's chain of loads (9-point, us by rows 1 / 2
+      // / 8, k_galerkin: 129^2 -> 65^2 5.1 / 8.1 / 25.9, 6.0; 385^2 11.2 / 13.3 / 26.2, 14.3; 513^2 14.5 / 13.4
+      // / 26.2, 18.6; 1025^2 52.6 / 47.1 / 63.3, 60.3; 4097^2 742 / 662 / 618, 906)
       const int gx = (C.nx + kGalCols - 1) / kGalCols;
-      const int rows = (long long)gx * nyrc > 8LL * 152 * 16 ? 8 : 2;
+      const long long warps = (long long)gx * nyrc;  // of one row each
+      const int rows = warps <= 12 * 152 ? 1 : warps <= 128 * 152 ? 2 : 8;
       const dim3 g(gx, (nyrc + 4 * rows - 1) / (4 * rows));
       if (F.five_point)
         k_galerkin_rows<true><<<g, 128, 0, s>>>(lvl_of(F), C.nx, C.ny, nyrc, C.pitch, rows, C.cE, C.cN, C.cNE, C.cNW,
