@@ -594,6 +594,11 @@ __global__ void __launch_bounds__(128, 5) k_galerkin_rows(Lvl<double> F, int nxc
   }
 }
 
+// INT: conversions on the integer pipe (mg_common.cuh) instead of the conversion instruction, whose time
+// on the FP64 pipe is about that of the copy in HBM: faster where the arrays stay in L2 (us, INT against
+// the instruction: 513^2 3.5, 4.7; 1025^2 9.4, 12.6), slower on smaller and larger ones (129^2 2.5, 1.95;
+// 2049^2 63.8, 47.4).
+template <bool INT>
 __global__ void k_op_to_f32(int nx, int nyr, int ps, int pd, const double* __restrict__ a0,
                             const double* __restrict__ a1, const double* __restrict__ a2,
                             const double* __restrict__ a3, const double* __restrict__ a4,
@@ -603,13 +608,14 @@ __global__ void k_op_to_f32(int nx, int nyr, int ps, int pd, const double* __res
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= nx || j >= nyr) return;
   const size_t s = (size_t)j * ps + i, d = (size_t)j * pd + i;
-  b0[d] = narrow(a0[s]);
-  b1[d] = narrow(a1[s]);
-  b2[d] = five ? 0.0f : narrow(a2[s]);  // a 5-point operator's NE / NW are zero: not read
-  b3[d] = five ? 0.0f : narrow(a3[s]);
-  const float dg = narrow(a4[s]);
+  auto f32 = [](double v) { return INT ? narrow(v) : (float)v; };
+  b0[d] = f32(a0[s]);
+  b1[d] = f32(a1[s]);
+  b2[d] = five ? 0.0f : f32(a2[s]);  // a 5-point operator's NE / NW are zero: not read
+  b3[d] = five ? 0.0f : f32(a3[s]);
+  const float dg = f32(a4[s]);
   b4[d] = dg;
-  b5[d] = dinv_f32 ? 1.0f / dg : narrow(a5[s]);  // dinv_f32: reciprocal of the FP32 diagonal
+  b5[d] = dinv_f32 ? 1.0f / dg : f32(a5[s]);  // dinv_f32: reciprocal of the FP32 diagonal
 }
 
 // Dense matrix of the coarsest level's unknowns, inverted by Gauss-Jordan elimination
@@ -873,7 +879,9 @@ cudaError_t launch_op_to_f64(const OpF32& A, const OpF64& B, cudaStream_t s) {
 cudaError_t launch_op_to_f32(const OpF64& A, const OpF32& B, cudaStream_t s, bool dinv_f32) {
   const int nyr = rows_stored(A.ny, A.periodic);
   dim3 b(32, 8);
-  k_op_to_f32<<<grid2(A.nx, nyr, b), b, 0, s>>>(A.nx, nyr, A.pitch, B.pitch, A.cE, A.cN, A.cNE,
+  const long long nodes = (long long)A.nx * nyr;
+  const auto f = nodes >= 100000 && nodes <= 2000000 ? k_op_to_f32<true> : k_op_to_f32<false>;
+  f<<<grid2(A.nx, nyr, b), b, 0, s>>>(A.nx, nyr, A.pitch, B.pitch, A.cE, A.cN, A.cNE,
                                                 A.cNW, A.diag, A.dinv, B.cE, B.cN, B.cNE, B.cNW,
                                                 B.diag, B.dinv, A.five_point, dinv_f32 ? 1 : 0);
   return cudaGetLastError();
