@@ -399,7 +399,7 @@ cudaError_t launch_smooth_block(const Op<T>& A, const T* xin, T* xout, const T* 
   using N32 = std::integral_constant<int, 32>;
   if constexpr (sizeof(T) == 4) {
     // tall tiles (64 rows) where they fill the GPU, half as tall ones on small levels
-    const bool tall = (long long)A.nx * nyr > 48LL * 16 * 152;
+    const bool tall = (long long)A.nx * nyr > 48LL * 16 * kSMs;
     if (ns == 2) return tall ? go(Two(), N32(), N32()) : go(Two(), N32(), N16());
     return tall ? go(One(), N32(), N32()) : go(One(), N32(), N16());
   } else {

@@ -771,7 +771,7 @@ static cudaError_t assemble_pass(const OpF64& A, const OpF32* B, double hx, doub
   // 2049^2 165 / 158 / 154, 195)
   const int gx = (A.nx + kAsmCols - 1) / kAsmCols;
   const long long warps = (long long)gx * nyr;  // of one row each
-  const int rows = warps <= 40 * 152 ? 1 : warps <= 240 * 152 ? 2 : 8;
+  const int rows = warps <= 40 * kSMs ? 1 : warps <= 240 * kSMs ? 2 : 8;
   dim3 b(32, 8), g(gx, (nyr + 8 * rows - 1) / (8 * rows));
   k_assemble_pass<FIVE><<<g, b, 0, s>>>(
       A.nx, A.ny, nyr, A.periodic, A.pitch, -0.5 * (1.0 / (hx * hx)), -0.5 * (1.0 / (hy * hy)), 1.0 / (4.0 * hx * hy), exx,
@@ -828,7 +828,7 @@ cudaError_t launch_galerkin(const Op<T>& F, const Op<T>& C, cudaStream_t s) {
       // / 26.2, 18.6; 1025^2 52.6 / 47.1 / 63.3, 60.3; 4097^2 742 / 662 / 618, 906)
       const int gx = (C.nx + kGalCols - 1) / kGalCols;
       const long long warps = (long long)gx * nyrc;  // of one row each
-      const int rows = warps <= 12 * 152 ? 1 : warps <= 128 * 152 ? 2 : 8;
+      const int rows = warps <= 12 * kSMs ? 1 : warps <= 128 * kSMs ? 2 : 8;
       const dim3 g(gx, (nyrc + 4 * rows - 1) / (4 * rows));
       if (F.five_point)
         k_galerkin_rows<true><<<g, 128, 0, s>>>(lvl_of(F), C.nx, C.ny, nyrc, C.pitch, rows, C.cE, C.cN, C.cNE, C.cNW,

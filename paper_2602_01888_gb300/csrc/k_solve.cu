@@ -570,7 +570,7 @@ dim3 red_grid(int nx, int nyr) {
   const int gx = (nx + kNT - 1) / kNT;
   int gy = kRedBlocks / gx;
   if (gy < 1) gy = 1;
-  const int fewest = (152 + gx - 1) / gx, spread = (nyr + 3) / 4;
+  const int fewest = (kSMs + gx - 1) / gx, spread = (nyr + 3) / 4;
   const int most = spread > fewest ? spread : (fewest < nyr ? fewest : nyr);
   if (gy > most) gy = most;
   return dim3(gx, gy);

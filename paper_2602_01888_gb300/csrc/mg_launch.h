@@ -7,6 +7,7 @@
 
 namespace mg {
 
+constexpr int kSMs = 152;             // SMs of a GB300, for the rules that split work by size
 constexpr int kCoarseMax = 256;      // unknowns of the coarsest level (dense inverse)
 constexpr int kCoarseThreads = 256;  // threads of the single-CTA coarsest solve
 constexpr int kCoarseFactorThreads = 1024;

@@ -85,7 +85,7 @@ inline long long block_nodes_f64() {
   static long long v = -1;
   if (v < 0) {
     const char* e = getenv("MG_BLOCK_NODES_F64");
-    v = e ? atoll(e) : 107008;
+    v = e ? atoll(e) : 2 * kSMs * 22 * 16;
   }
   return v;
 }
